@@ -459,13 +459,8 @@ int dsm_create(const dsm_layout* layout, uint32_t n, uint32_t tau, const dsm_hpa
         td.lam_global = t.wd ? hp->g_wd : 0.0f;
         td.kind = t.kind;
         td.tile_begin = static_cast<uint32_t>(h->tiles.size());
-        for (uint64_t o = 0; o < t.numel; o += kTile) {
-            TileDesc tl;
-            tl.start = off + o;
-            tl.len = static_cast<uint32_t>(t.numel - o < kTile ? t.numel - o : kTile);
-            tl.tensor = i;
-            h->tiles.push_back(tl);
-        }
+        const uint64_t count = (t.numel + kTile - 1) / kTile;
+        for (uint64_t c = 0; c < count; ++c) h->tiles.push_back(make_tile(off, t.numel, i, c));
         td.tile_end = static_cast<uint32_t>(h->tiles.size());
         td.pad = 0;
         off += t.numel;
@@ -643,7 +638,7 @@ int dsm_local_step_host_grads(dsm_handle* h, const void* src, dsm_stream_t strea
     const uint32_t chunks = static_cast<uint32_t>(h->ev_copied.size());
     for (uint32_t c = 0; c < chunks; ++c) {
         const uint32_t t0 = h->chunk_tile[c], t1 = h->chunk_tile[c + 1];
-        const uint64_t e0 = h->tiles[t0].start, e1 = h->tiles[t1 - 1].start + h->tiles[t1 - 1].len;
+        const uint64_t e0 = h->tiles[t0].start + h->tiles[t0].skip(), e1 = h->tiles[t1 - 1].start + h->tiles[t1 - 1].end();
         err = cudaMemcpy2DAsync(grad + e0 * es, h->al.d_stride * es, host + e0 * es, h->al.d * es, (e1 - e0) * es,
                                 h->n, cudaMemcpyHostToDevice, cs);
         if (err == cudaSuccess) err = cudaEventRecord(h->ev_copied[c], cs);

@@ -62,8 +62,11 @@ __host__ __device__ constexpr size_t fused_smem(bool adamw, bool bf16, int nw, i
             size_t(fused_glob_sets(adamw, nw)) * fused_globals(global) * 16) * kThreads;
 }
 
+// CTAs per SM: 4 up to n = 4 and 3 above, as many as the staging allows.  Left to itself the compiler gave the
+// global AdamW instantiations 111-212 registers for n > 4, 2 CTAs or 1: K6 for n = 6, bf16 gradients, 16.3 M
+// parameters took 436 us against 390 us with 3.
 template <bool kAdamW, bool kBf16, int NW, int kGlobal>
-__global__ void __launch_bounds__(kThreads) k_fused_last_global(Problem p, AdamScalars a, SgdmScalars sa,
+__global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global(Problem p, AdamScalars a, SgdmScalars sa,
                                                                 GlobalScalars g, int opts) {
     constexpr int kFusedDepth = fused_depth(kAdamW, NW);
     constexpr int kStates = fused_states(kAdamW), kGlobals = fused_globals(kGlobal);
@@ -199,40 +202,39 @@ __global__ void __launch_bounds__(kThreads) k_fused_last_global(Problem p, AdamS
             // this thread issued no copies for the tile; keep the group count in step
 #pragma unroll
             for (int w = 0; w < NW; ++w, ++it) issue(next_issue++);
-            const uint32_t e1 = min(e0 + kElemsPerThread, td.len);
-            for (uint32_t e = e0; e < e1; ++e) {
-                const uint64_t gj = td.start + e;
-                float x = p.x[gj], m = p.m[gj], d[NW];
+        }
+        if (uint32_t e; edge_element(td, e)) {
+            const uint64_t gj = td.start + e;
+            float x = p.x[gj], m = p.m[gj], d[NW];
 #pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    const uint64_t o = w * p.d_stride + gj;
-                    float xi = from_global ? x : p.X[o], mi = zero_state ? 0.f : p.opt_m[o];
-                    if (kAdamW) {
-                        float vi = zero_state ? 0.f : p.opt_v[o];
-                        adamw_elem(xi, mi, vi, load_grad1(p.grad, kBf16, o), a, lam_l);
-                        if (keep_state) p.opt_v[o] = vi;
-                    } else {
-                        sgdm_elem(xi, mi, load_grad1(p.grad, kBf16, o), sa);
-                    }
-                    if (keep_state) p.opt_m[o] = mi;
-                    d[w] = __fsub_rn(x, xi);
-                }
-                float r = 0.f;
-                if (kGlobal == kGlobalSign && g.sign_mode != 0)
-                    r = philox_unit(word_of(philox_block((gj >> 2) + g.philox_q0, g.philox_k0, g.philox_k1), gj & 3));
-                if (kGlobal == kGlobalRuntime) {
-                    global_elem_rt<NW>(x, m, d, g, lam_g, r, st);
-                } else if (kGlobal == kGlobalAdamW) {
-                    float v = p.gv[gj];
-                    global_elem<NW, 4>(x, m, v, d, NW, g, lam_g, r, st);
-                    p.gv[gj] = v;
+            for (int w = 0; w < NW; ++w) {
+                const uint64_t o = w * p.d_stride + gj;
+                float xi = from_global ? x : p.X[o], mi = zero_state ? 0.f : p.opt_m[o];
+                if (kAdamW) {
+                    float vi = zero_state ? 0.f : p.opt_v[o];
+                    adamw_elem(xi, mi, vi, load_grad1(p.grad, kBf16, o), a, lam_l);
+                    if (keep_state) p.opt_v[o] = vi;
                 } else {
-                    float unused = 0.f;
-                    global_elem<NW, 0>(x, m, unused, d, NW, g, lam_g, r, st);
+                    sgdm_elem(xi, mi, load_grad1(p.grad, kBf16, o), sa);
                 }
-                p.x[gj] = x;
-                p.m[gj] = m;
+                if (keep_state) p.opt_m[o] = mi;
+                d[w] = __fsub_rn(x, xi);
             }
+            float r = 0.f;
+            if (kGlobal == kGlobalSign && g.sign_mode != 0)
+                r = philox_unit(word_of(philox_block((gj >> 2) + g.philox_q0, g.philox_k0, g.philox_k1), gj & 3));
+            if (kGlobal == kGlobalRuntime) {
+                global_elem_rt<NW>(x, m, d, g, lam_g, r, st);
+            } else if (kGlobal == kGlobalAdamW) {
+                float v = p.gv[gj];
+                global_elem<NW, 4>(x, m, v, d, NW, g, lam_g, r, st);
+                p.gv[gj] = v;
+            } else {
+                float unused = 0.f;
+                global_elem<NW, 0>(x, m, unused, d, NW, g, lam_g, r, st);
+            }
+            p.x[gj] = x;
+            p.m[gj] = m;
         }
         const uint32_t next = ti + gridDim.x;
         if (next >= p.num_tiles || p.tiles[next].tensor != td.tensor) {  // uniform across the CTA

@@ -33,27 +33,37 @@ namespace {
 // Kernels
 // ---------------------------------------------------------------------------
 
-// Initial state: x (hash init by tensor kind, or as already copied) and every replica = x.
+// Initial value of element gi (hash init by tensor kind).
+__device__ __forceinline__ float init_value(uint32_t kind, float u) {
+    if (kind == 0) return __fmul_rn(0.02f, __fsub_rn(__fmul_rn(2.0f, u), 1.0f));
+    return kind == 2 ? 1.0f : 0.0f;
+}
+
+// Initial state: x (hash init by tensor kind, or as already copied) and every replica = x.  Also the reset of
+// the replicas that a lazy round left pending.  Bound by its writes: n 16-byte stores per group of 4 elements
+// (with 4-byte accesses, 16 bytes apart between threads, it took 1.26 ms on GPT-2 S with n = 4, 2.5 GB).
 __global__ void __launch_bounds__(kThreads) k_init(Problem p, uint64_t key_init, int from_hash) {
+    const uint32_t e0 = threadIdx.x * kElemsPerThread;
     for (uint32_t ti = blockIdx.x; ti < p.num_tiles; ti += gridDim.x) {
         const TileDesc td = p.tiles[ti];
         const uint32_t kind = p.tensors[td.tensor].kind;
-        const uint32_t e0 = threadIdx.x * kElemsPerThread;
-        const uint32_t e1 = min(e0 + kElemsPerThread, td.len);
-        for (uint32_t e = e0; e < e1; ++e) {
-            const uint64_t gi = td.start + e;
-            float v;
+        if (vector_ok(td, e0)) {
+            const uint64_t gi = td.start + e0;
+            float v[4];
             if (from_hash) {
-                if (kind == 0) {
-                    const float u = hash_uniform(key_init, gi);
-                    v = __fmul_rn(0.02f, __fsub_rn(__fmul_rn(2.0f, u), 1.0f));
-                } else {
-                    v = (kind == 2) ? 1.0f : 0.0f;
-                }
-                p.x[gi] = v;
+                const uint64_t h0 = sm64_output(key_init, (gi >> 1) + 1), h1 = sm64_output(key_init, (gi >> 1) + 2);
+                v[0] = init_value(kind, draw_even(h0)); v[1] = init_value(kind, draw_odd(h0));
+                v[2] = init_value(kind, draw_even(h1)); v[3] = init_value(kind, draw_odd(h1));
+                store4(p.x + gi, v);
             } else {
-                v = p.x[gi];
+                load4(p.x + gi, v);
             }
+            for (uint32_t w = 0; w < p.n; ++w) store4(p.X + w * p.d_stride + gi, v);
+        }
+        if (uint32_t e; edge_element(td, e)) {
+            const uint64_t gi = td.start + e;
+            const float v = from_hash ? init_value(kind, hash_uniform(key_init, gi)) : p.x[gi];
+            if (from_hash) p.x[gi] = v;
             for (uint32_t w = 0; w < p.n; ++w) p.X[w * p.d_stride + gi] = v;
         }
     }
@@ -113,7 +123,7 @@ __device__ __forceinline__ void grad_fill_groups(const Problem& p, const GradKey
     }
 }
 
-// Element-by-element fill (tile starts that are not 4-aligned, ragged tails).
+// Element-by-element fill (a tensor's partial groups).
 template <bool kBf16>
 __device__ __forceinline__ void grad_fill_elem(const Problem& p, const GradKeys& k, uint64_t gi, float s, float s2) {
     const float a = step_term(s, hash_uniform(k.step, gi));
@@ -135,20 +145,20 @@ __global__ void __launch_bounds__(kFillThreads) k_grad_fill(Problem p, GradKeys 
         // one multiplication per draw where both scales allow it (see centred_even)
         const bool pre = fabsf(s) >= kMinPrescaled && fabsf(s2) >= kMinPrescaled;
         const float sp = __fmul_rn(s, kTwoPowM24), sp2 = __fmul_rn(s2, kTwoPowM24);
-        const bool aligned = (td.start & 3u) == 0;
-        if (aligned && td.len == kTile) {  // a full tile (uniform across the CTA)
+        if (td.skip() == 0 && td.end() == kTile) {  // a full tile (uniform across the CTA)
             const uint64_t gi0 = td.start + threadIdx.x * 4;
             if (pre) grad_fill_groups<kBf16, true, kFillGroups, kStride>(p, k, gi0, sp, sp2);
             else grad_fill_groups<kBf16, false, kFillGroups, kStride>(p, k, gi0, s, s2);
             continue;
         }
-        for (uint32_t e0 = threadIdx.x * 4; e0 < td.len; e0 += kStride) {  // a ragged tile, group by group
-            if (aligned && e0 + 4 <= td.len) {
+        for (uint32_t e0 = threadIdx.x * 4; e0 < td.end(); e0 += kStride) {  // a ragged tile, group by group
+            if (vector_ok(td, e0)) {
                 if (pre) grad_fill_groups<kBf16, true, 1, kStride>(p, k, td.start + e0, sp, sp2);
                 else grad_fill_groups<kBf16, false, 1, kStride>(p, k, td.start + e0, s, s2);
             } else {
-                const uint32_t e1 = min(e0 + 4u, td.len);
-                for (uint32_t e = e0; e < e1; ++e) grad_fill_elem<kBf16>(p, k, td.start + e, s, s2);
+                const uint32_t e1 = min(e0 + 4u, td.end());
+                for (uint32_t e = max(e0, td.skip()); e < e1; ++e)
+                    grad_fill_elem<kBf16>(p, k, td.start + e, s, s2);
             }
         }
     }
@@ -280,8 +290,9 @@ __device__ __forceinline__ void global_vec_generic(const Problem& p, const Globa
 // grid of G CTAs, tile t is a CTA's last tile of its tensor exactly when
 // t + G lies beyond the tensor, so the partials of a tensor are its last
 // min(G, tiles) tiles, which K5 sums.
+// CTAs per SM: what the double-buffered replicas leave room for (4 for n = 1, 3 up to n = 4, 2 above).
 template <int NW, int MODE>
-__global__ void __launch_bounds__(kThreads) k_global(Problem p, GlobalScalars g) {
+__global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_global(Problem p, GlobalScalars g) {
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
     constexpr int W = NW > 0 ? NW : 1;
     uint32_t ti = blockIdx.x;
@@ -345,10 +356,8 @@ __global__ void __launch_bounds__(kThreads) k_global(Problem p, GlobalScalars g)
             }
         } else if (NW == 0 && vector_ok(td, e0)) {
             global_vec_generic<MODE>(p, g, lam, td.start + e0, st);
-        } else {
-            const uint32_t e1 = min(e0 + kElemsPerThread, td.len);
-            for (uint32_t e = e0; e < e1; ++e) global_elem_generic<MODE>(p, g, lam, td.start + e, st);
         }
+        if (uint32_t e; edge_element(td, e)) global_elem_generic<MODE>(p, g, lam, td.start + e, st);
         if (next >= p.num_tiles || nt.tensor != td.tensor) {  // uniform across the CTA
             reduce_stats(st, p.partials + ti);
             st = ThreadStats();

@@ -18,7 +18,7 @@ namespace {
 struct LocalItem {
     uint64_t base;   // w * d_stride + tile start
     uint64_t start;  // tile start (offset in x)
-    uint32_t len;
+    uint32_t ends;   // of the tile (its partial groups' elements)
     float lam;
     bool vec;
 };
@@ -56,7 +56,7 @@ __device__ __forceinline__ LocalItem local_item(const Problem& p, uint32_t w, ui
     LocalItem it;
     it.base = w * p.d_stride + td.start;
     it.start = td.start;
-    it.len = td.len;
+    it.ends = td.ends;
     it.lam = local_lam ? p.tensors[td.tensor].lam_local : 0.f;
     it.vec = vector_ok(td, e0);
     return it;
@@ -107,15 +107,13 @@ __global__ void __launch_bounds__(kThreads) k_local_adamw(Problem p, AdamScalars
             store4(p.X + cur.base + e0, cx);
             store4(p.opt_m + cur.base + e0, cm);
             store4(p.opt_v + cur.base + e0, cv);
-        } else {
-            const uint32_t e1 = min(e0 + kElemsPerThread, cur.len);
-            for (uint32_t e = e0; e < e1; ++e) {
-                const uint64_t i = cur.base + e;
-                float xs = kFromGlobal ? p.x[cur.start + e] : p.X[i];
-                float ms = kZeroState ? 0.f : p.opt_m[i], vs = kZeroState ? 0.f : p.opt_v[i];
-                adamw_elem(xs, ms, vs, load_grad1(p.grad, kBf16, i), a, cur.lam);
-                p.X[i] = xs; p.opt_m[i] = ms; p.opt_v[i] = vs;
-            }
+        }
+        if (uint32_t e; edge_element(TileDesc{0, cur.ends, 0}, e)) {
+            const uint64_t i = cur.base + e;
+            float xs = kFromGlobal ? p.x[cur.start + e] : p.X[i];
+            float ms = kZeroState ? 0.f : p.opt_m[i], vs = kZeroState ? 0.f : p.opt_v[i];
+            adamw_elem(xs, ms, vs, load_grad1(p.grad, kBf16, i), a, cur.lam);
+            p.X[i] = xs; p.opt_m[i] = ms; p.opt_v[i] = vs;
         }
     }
 }
@@ -156,14 +154,12 @@ __global__ void __launch_bounds__(kThreads) k_local_sgdm(Problem p, SgdmScalars 
             for (int j = 0; j < 4; ++j) sgdm_elem(cx[j], cb[j], cg[j], a);
             store4(p.X + cur.base + e0, cx);
             store4(p.opt_m + cur.base + e0, cb);
-        } else {
-            const uint32_t e1 = min(e0 + kElemsPerThread, cur.len);
-            for (uint32_t e = e0; e < e1; ++e) {
-                const uint64_t i = cur.base + e;
-                float xs = kFromGlobal ? p.x[cur.start + e] : p.X[i], bs = kZeroState ? 0.f : p.opt_m[i];
-                sgdm_elem(xs, bs, load_grad1(p.grad, kBf16, i), a);
-                p.X[i] = xs; p.opt_m[i] = bs;
-            }
+        }
+        if (uint32_t e; edge_element(TileDesc{0, cur.ends, 0}, e)) {
+            const uint64_t i = cur.base + e;
+            float xs = kFromGlobal ? p.x[cur.start + e] : p.X[i], bs = kZeroState ? 0.f : p.opt_m[i];
+            sgdm_elem(xs, bs, load_grad1(p.grad, kBf16, i), a);
+            p.X[i] = xs; p.opt_m[i] = bs;
         }
     }
 }

@@ -91,12 +91,7 @@ __global__ void __launch_bounds__(kThreads) k_noalloc_tile_table(unsigned char* 
             else hi = mid;
         }
         const TensorDesc& T = t[lo - 1];
-        const uint64_t o = uint64_t(ti - T.tile_begin) * kTile;
-        TileDesc d;
-        d.start = T.off + o;
-        d.len = static_cast<uint32_t>(T.numel - o < kTile ? T.numel - o : kTile);
-        d.tensor = lo - 1;
-        tiles[ti] = d;
+        tiles[ti] = make_tile(T.off, T.numel, lo - 1, ti - T.tile_begin);
     }
 }
 

@@ -117,6 +117,39 @@ def test_global_variants_bitexact(layout_name, name, hp, n, tau, fused):
     run.close()
 
 
+def _every_offset(sizes):
+    """Tensors of the given sizes, each at every offset modulo 4 (one-element tensors in between shift them)."""
+    tensors, off = [], 0
+    for s in sizes:
+        for r in range(4):
+            while off % 4 != r:
+                tensors.append(W.Tensor("shift", 1, W.KIND_BIAS, 1e-3, wd=0))
+                off += 1
+            tensors.append(W.Tensor(f"{s}at{r}", s, W.KIND_WEIGHT, 1e-2))
+            off += s
+    return tuple(tensors)
+
+
+@pytest.mark.parametrize("fused", [False, True], ids=["unfused", "fused"])
+@pytest.mark.parametrize("name,hp,n", [("adamw-bf16-n2", dataclasses.replace(ADAMW, grad_dtype=W.BF16), 2),
+                                       ("sgdm-rsign-n3", SGDM, 3),
+                                       ("gadamw-n9", dataclasses.replace(ADAMW, global_mode=W.GLOBAL_ADAMW), 9)],
+                         ids=lambda v: v if isinstance(v, str) else "")
+def test_partial_groups_bitexact(name, hp, n, fused):
+    """Tensors whose first and last groups of 4 elements are partial in every way: tiny tensors inside one group, and
+    sizes around the tile (up to 3 elements of the last group lie beyond a tile of 1024)."""
+    tensors = _every_offset([1, 2, 3, 4, 5, 7, 1020, 1021, 1023, 1024, 1025, 2048, 2051])
+    hp = dataclasses.replace(hp, flags=W.FLAG_FUSED_ROUND if fused else 0)
+    run = dsm.DistributedSignMomentum(tensors, n, 2, hp)
+    ora = O.OracleRun(tensors, n, 2, hp, with_stats=True)
+    for _ in range(2):
+        stats = run.synthetic_round(with_stats=True)
+        ora.run_round()
+        compare_state(run, ora)
+        compare_stats(stats, ora.last_stats, n)
+    run.close()
+
+
 FUSED = [
     ("adamw-f32-n4-t3", ADAMW, 4, 3),
     ("adamw-bf16-n8-t2", dataclasses.replace(ADAMW, grad_dtype=W.BF16), 8, 2),
