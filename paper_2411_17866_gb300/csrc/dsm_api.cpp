@@ -291,6 +291,9 @@ void next_local_scalars(const dsm_handle* h, AdamScalars* a, SgdmScalars* sa, do
         a->bc2 = float(1.0 - *nb2);
         a->lr = h->gamma;
         a->eps = h->hp.eps;
+        a->rbc1 = float(1.0 / double(a->bc1));
+        a->rbc2 = float(1.0 / double(a->bc2));
+        a->newton = a->bc1 >= 0x1p-24f && a->bc2 >= 0x1p-24f && a->eps <= 0x1p60f;
     } else {
         sa->mu = h->hp.mu;
         sa->lr = h->gamma;

@@ -162,10 +162,10 @@ __global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global
                     take(reinterpret_cast<const float4*>(grad_slot(it)), gr);
                 }
                 const uint64_t o = w * p.d_stride + gi;
+                if (kAdamW) adamw_group(xi, mi, vi, gr, a, lam_l);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    if (kAdamW) adamw_elem(xi[j], mi[j], vi[j], gr[j], a, lam_l);
-                    else sgdm_elem(xi[j], mi[j], gr[j], sa);
+                    if (!kAdamW) sgdm_elem(xi[j], mi[j], gr[j], sa);
                     dif[w][j] = __fsub_rn(x[j], xi[j]);
                 }
                 if (keep_state) {

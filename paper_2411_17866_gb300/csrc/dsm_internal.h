@@ -118,6 +118,8 @@ struct AdamScalars {
     float b2, omb2;        // beta2, 1 - beta2
     float bc1, bc2;        // 1 - beta1^j, 1 - beta2^j
     float lr, eps;
+    float rbc1, rbc2;      // 1/bc1 and 1/bc2, correctly rounded
+    int newton;            // the scalars lie in the ranges that adamw_group() needs for its Newton forms
 };
 
 struct SgdmScalars {

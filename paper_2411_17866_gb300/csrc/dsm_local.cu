@@ -102,8 +102,7 @@ __global__ void __launch_bounds__(kThreads) k_local_adamw(Problem p, AdamScalars
             }
         }
         if (cur.vec) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) adamw_elem(cx[j], cm[j], cv[j], cg[j], a, cur.lam);
+            adamw_group(cx, cm, cv, cg, a, cur.lam);
             store4(p.X + cur.base + e0, cx);
             store4(p.opt_m + cur.base + e0, cm);
             store4(p.opt_v + cur.base + e0, cv);
@@ -168,12 +167,14 @@ __global__ void __launch_bounds__(kThreads) k_local_sgdm(Problem p, SgdmScalars 
 
 cudaError_t query_local_shape(const Problem& p, LaunchShape* out) {
     const int sms = out->sms;
-    // The AdamW step fits 4 CTAs per SM.  With fp32 gradients it streams better with 3 (GB300, GPT-2 S,
-    // n = 4: 1.00 of the copy bandwidth with 3, 0.95 with 4); with bf16 gradients 4 are better
-    // (GPT-2 M, n = 8: 0.97 with 4, 0.90 with 3; GPT-2 XL, n = 4: 0.96 with 4, 0.87 with 3).
-    const int kAdamwCtasPerSm = p.grad_bf16 ? 4 : 3;
+    // The AdamW step fits 5 CTAs per SM; it streams best with about as many bytes in flight as the memory takes
+    // (GB300, us a step).  From the replicas, fp32 gradients, GPT-2 S with n = 4: 2071 / 2033 / 2056 / 2111 with 2.75 /
+    // 3 / 3.25 / 4 CTAs per SM; bf16: 2010 / 1935 / 1907 / 1954 with 2.75 / 3 / 3.5 / 4.  From x (a round of two steps,
+    // 184 M parameters, n = 8) fp32: 11279 / 11060 / 11122 with 3 / 3.5 / 4; bf16: 10764 / 10511 / 10294 / 10639 with
+    // 3 / 3.5 / 4 / 4.5.
+    const int adamw_ctas = p.grad_bf16 ? 7 * sms / 2 : 3 * sms, adamw_ctas_from_x = p.grad_bf16 ? 4 * sms : 7 * sms / 2;
     out->grid_adamw = std::min(p.grad_bf16 ? grid_for(k_local_adamw<true, false, false>, sms)
-                                           : grid_for(k_local_adamw<false, false, false>, sms), kAdamwCtasPerSm * sms);
+                                           : grid_for(k_local_adamw<false, false, false>, sms), adamw_ctas);
     // The SGD-momentum step fits 6 CTAs per SM, but 4 stream better (GB300, GPT-2 L layout, n = 8:
     // 0.96 of the copy bandwidth with 4, 0.91 with 6, 0.91 with 3), as many as the AdamW step holds.
     constexpr int kSgdmCtasPerSm = 4;
@@ -182,7 +183,7 @@ cudaError_t query_local_shape(const Problem& p, LaunchShape* out) {
     {  // the from-x variants (first local step after a lazy reset)
         out->grid_adamw_from_x = std::min(p.grad_bf16 ? grid_for(k_local_adamw<true, true, false>, sms)
                                                       : grid_for(k_local_adamw<false, true, false>, sms),
-                                          kAdamwCtasPerSm * sms);
+                                          adamw_ctas_from_x);
         out->grid_sgdm_from_x = std::min(p.grad_bf16 ? grid_for(k_local_sgdm<true, true, false>, sms)
                                                      : grid_for(k_local_sgdm<false, true, false>, sms),
                                          kSgdmCtasPerSm * sms);

@@ -150,6 +150,64 @@ def test_partial_groups_bitexact(name, hp, n, fused):
     run.close()
 
 
+@pytest.mark.parametrize("hp", [ADAMW, dataclasses.replace(ADAMW, grad_dtype=W.BF16, b1=0.0, b2=0.0),
+                                dataclasses.replace(ADAMW, b1=0.9999999, b2=0.99999994, eps=1e-30),
+                                dataclasses.replace(ADAMW, eps=1e20)],
+                         ids=["defaults", "bf16-betas-0", "bias-corrections-2^-24", "eps-beyond-2^60"])
+@pytest.mark.parametrize("n", [1, 3])
+def test_adamw_over_the_whole_range_bitexact(n, hp):
+    """AdamW on moments and gradients of every magnitude, zeros, denormals and infinities among them: whole groups of 4
+    inside the ranges of the branch-free division, whole groups outside and mixed ones, at both ends of each range."""
+    d = 1 << 16
+    rng = np.random.default_rng(3)
+    edges = np.float32([0.0, -0.0, 1e-45, 2.0 ** -126, 2.0 ** -101, 2.0 ** -100, 2.0 ** -61, 2.0 ** -60, 2.0 ** 50,
+                        2.0 ** 51, 2.0 ** 100, 2.0 ** 101, 3e38, np.inf])
+
+    def values(lo, hi, signed):
+        v = (rng.uniform(1, 2, d) * 2.0 ** rng.integers(lo, hi, d)).astype(np.float32)
+        some = rng.random(d) < 0.05
+        v[some] = edges[rng.integers(0, edges.size, d)[some]]
+        inside = np.repeat(rng.random(d // 4) < 0.3, 4)      # whole groups of usual sizes
+        v[inside] = (rng.uniform(1, 2, d) * 2.0 ** rng.integers(-30, -5, d)).astype(np.float32)[inside]
+        return v * np.where(rng.random(d) < 0.5, -1, 1).astype(np.float32) if signed else v
+
+    tensors = (W.Tensor("t", d, W.KIND_WEIGHT, 1e-3),)
+    for fused in (False, True):
+        hpf = dataclasses.replace(hp, flags=W.FLAG_FUSED_ROUND if fused else 0)
+        run, ora = dsm.DistributedSignMomentum(tensors, n, 1, hpf), O.OracleRun(tensors, n, 1, hpf)
+        grads = []
+        for i in range(n):
+            m, v = values(-149, 127, True), values(-149, 127, False)
+            run.write(dsm.BUF_OPT_M, torch.from_numpy(m), worker=i)
+            run.write(dsm.BUF_OPT_V, torch.from_numpy(v), worker=i)
+            ora.opt_m[i][:], ora.opt_v[i][:] = m, v
+            g = torch.from_numpy(values(-75, 64, True))
+            g = g.bfloat16() if hp.grad_dtype == W.BF16 else g
+            run.grad_view(i).copy_(g)
+            grads.append(g.float().numpy())
+        run.local_step()
+        with np.errstate(all="ignore"):
+            ora.local_step(grads)
+        for i in range(n if not fused else 0):
+            same_but_for_nan(run.read(dsm.BUF_REPLICA, i).numpy(), ora.X[i], f"replica {i}")
+        run.global_step()
+        with np.errstate(all="ignore"):
+            ora.global_step()
+        same_but_for_nan(run.read(dsm.BUF_X).numpy(), ora.x, "x")
+        same_but_for_nan(run.read(dsm.BUF_M).numpy(), ora.m, "m")
+        for i in range(n):
+            same_but_for_nan(run.read(dsm.BUF_OPT_M, i).numpy(), ora.opt_m[i], f"opt_m {i}")
+            same_but_for_nan(run.read(dsm.BUF_OPT_V, i).numpy(), ora.opt_v[i], f"opt_v {i}")
+        run.close()
+
+
+def same_but_for_nan(got, want, what):
+    got, want = np.asarray(got), np.asarray(want, np.float32)
+    nan = np.isnan(want)
+    assert np.array_equal(np.isnan(got), nan), f"{what}: NaN positions differ"
+    assert_bitexact(got[~nan], want[~nan], what)
+
+
 FUSED = [
     ("adamw-f32-n4-t3", ADAMW, 4, 3),
     ("adamw-bf16-n8-t2", dataclasses.replace(ADAMW, grad_dtype=W.BF16), 8, 2),
