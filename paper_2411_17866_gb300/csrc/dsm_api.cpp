@@ -489,6 +489,7 @@ int dsm_create(const dsm_layout* layout, uint32_t n, uint32_t tau, const dsm_hpa
     p.partials = reinterpret_cast<StatPartial*>(A + al.off_partials);
     p.stats = reinterpret_cast<TensorStats*>(A + al.off_stats);
 
+    p.early = true;
     DeviceGuard guard(h->device);
     if (guard.err != cudaSuccess) {
         delete h;

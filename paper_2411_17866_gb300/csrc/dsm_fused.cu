@@ -46,9 +46,8 @@ cudaError_t launch_fused_last_global(const Problem& p, const LaunchShape& ls, co
     const int grid = clamp_grid(ls.grid_fused, p.num_tiles);
     *grid_used = static_cast<uint32_t>(grid);
     if (grid == 0) return cudaSuccess;
-    fused_kernel_for(p, p.opt_v != nullptr)<<<grid, kThreads, fused_smem_for(p, p.opt_v != nullptr), s>>>(
-        p, a, sa, g, opts);
-    return cudaGetLastError();
+    const bool adamw = p.opt_v != nullptr;
+    return launch(fused_kernel_for(p, adamw), grid, kThreads, fused_smem_for(p, adamw), s, p.early, p, a, sa, g, opts);
 }
 
 }  // namespace dsm

@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global
         v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
     };
     uint32_t next_issue = 0;
+    wait_previous();
     for (int k = 0; k < kFusedDepth; ++k) issue(next_issue++);
     ThreadStats st;
     uint32_t it = 0;

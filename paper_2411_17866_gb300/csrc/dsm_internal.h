@@ -108,6 +108,8 @@ struct Problem {
     float* opt_v;          // [n][d_stride] (AdamW only)
     void* grad;            // [n][d_stride], fp32 or bf16
     int grad_bf16;
+    bool early;            // kernels may start before the one before them has ended (wait_previous() in
+                           // dsm_device.cuh): the tables above are not written by a kernel just before
     StatPartial* partials; // [num_tiles]; only each CTA's last tile of a tensor is written
     TensorStats* stats;    // [num_tensors]
 };

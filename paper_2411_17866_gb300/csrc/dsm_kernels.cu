@@ -44,6 +44,7 @@ __device__ __forceinline__ float init_value(uint32_t kind, float u) {
 // (with 4-byte accesses, 16 bytes apart between threads, it took 1.26 ms on GPT-2 S with n = 4, 2.5 GB).
 __global__ void __launch_bounds__(kThreads) k_init(Problem p, uint64_t key_init, int from_hash) {
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
+    wait_previous();
     for (uint32_t ti = blockIdx.x; ti < p.num_tiles; ti += gridDim.x) {
         const TileDesc td = p.tiles[ti];
         const uint32_t kind = p.tensors[td.tensor].kind;
@@ -138,6 +139,7 @@ __device__ __forceinline__ void grad_fill_elem(const Problem& p, const GradKeys&
 template <bool kBf16>
 __global__ void __launch_bounds__(kFillThreads) k_grad_fill(Problem p, GradKeys k) {
     constexpr uint32_t kStride = 4 * kFillThreads;  // elements between a thread's groups
+    wait_previous();
     for (uint32_t ti = blockIdx.x; ti < p.num_tiles; ti += gridDim.x) {
         const TileDesc td = p.tiles[ti];
         const TensorDesc& T = p.tensors[td.tensor];
@@ -296,9 +298,9 @@ __global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
     constexpr int W = NW > 0 ? NW : 1;
     uint32_t ti = blockIdx.x;
-    if (ti >= p.num_tiles) return;
     TileDesc nt = p.tiles[ti];
     bool nvec = NW > 0 && vector_ok(nt, e0);
+    wait_previous();
     float x[4], m[4], v[4] = {0.f, 0.f, 0.f, 0.f}, r[W][4];
     ThreadStats st;
     if (nvec) {
@@ -371,6 +373,7 @@ __global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4
 __global__ void __launch_bounds__(kThreads) k_stats(Problem p, uint32_t producer_grid) {
     const uint32_t T = blockIdx.x;
     const TensorDesc td = p.tensors[T];
+    wait_previous();
     double a = 0.0, b = 0.0;
     unsigned long long c0 = 0, c1 = 0, c2 = 0, c3 = 0;
     const uint32_t first =
@@ -470,16 +473,13 @@ cudaError_t query_launch_shape(const Problem& p, LaunchShape* out) {
 cudaError_t launch_init(const Problem& p, const LaunchShape& ls, uint64_t key_init, int from_hash, cudaStream_t s) {
     const int grid = clamp_grid(ls.grid_init, p.num_tiles);
     if (grid == 0) return cudaSuccess;
-    k_init<<<grid, kThreads, 0, s>>>(p, key_init, from_hash);
-    return cudaGetLastError();
+    return launch(k_init, grid, kThreads, 0, s, false, p, key_init, from_hash);
 }
 
 cudaError_t launch_grad_fill(const Problem& p, const LaunchShape& ls, const GradKeys& k, cudaStream_t s) {
     const int grid = clamp_grid(ls.grid_grad, p.num_tiles);
     if (grid == 0) return cudaSuccess;
-    if (p.grad_bf16) k_grad_fill<true><<<grid, kFillThreads, 0, s>>>(p, k);
-    else k_grad_fill<false><<<grid, kFillThreads, 0, s>>>(p, k);
-    return cudaGetLastError();
+    return launch(p.grad_bf16 ? k_grad_fill<true> : k_grad_fill<false>, grid, kFillThreads, 0, s, p.early, p, k);
 }
 
 cudaError_t launch_global(const Problem& p, const LaunchShape& ls, const GlobalScalars& g, cudaStream_t s,
@@ -487,14 +487,12 @@ cudaError_t launch_global(const Problem& p, const LaunchShape& ls, const GlobalS
     const int grid = clamp_grid(ls.grid_global, p.num_tiles);
     *grid_used = static_cast<uint32_t>(grid);
     if (grid == 0) return cudaSuccess;
-    global_kernel_for(p.n, p.global_mode)<<<grid, kThreads, 0, s>>>(p, g);
-    return cudaGetLastError();
+    return launch(global_kernel_for(p.n, p.global_mode), grid, kThreads, 0, s, p.early, p, g);
 }
 
 cudaError_t launch_stats(const Problem& p, uint32_t producer_grid, cudaStream_t s) {
     if (p.num_tensors == 0) return cudaSuccess;
-    k_stats<<<p.num_tensors, kThreads, 0, s>>>(p, producer_grid);
-    return cudaGetLastError();
+    return launch(k_stats, static_cast<int>(p.num_tensors), kThreads, 0, s, p.early, p, producer_grid);
 }
 
 }  // namespace dsm

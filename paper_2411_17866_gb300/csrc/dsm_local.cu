@@ -71,9 +71,9 @@ __global__ void __launch_bounds__(kThreads) k_local_adamw(Problem p, AdamScalars
     const uint32_t items = p.num_tiles * p.n;
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
     uint32_t item = blockIdx.x;
-    if (item >= items) return;
     ItemWalk<kFromGlobal> walk(p, item, gridDim.x);
     LocalItem nx = local_item(p, walk.w, walk.ti, e0, true);
+    wait_previous();
     float x[4], m[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f}, g[4];
     if (nx.vec) {
         load4(kFromGlobal ? p.x + nx.start + e0 : p.X + nx.base + e0, x);
@@ -124,9 +124,9 @@ __global__ void __launch_bounds__(kThreads) k_local_sgdm(Problem p, SgdmScalars 
     const uint32_t items = p.num_tiles * p.n;
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
     uint32_t item = blockIdx.x;
-    if (item >= items) return;
     ItemWalk<kFromGlobal> walk(p, item, gridDim.x);
     LocalItem nx = local_item(p, walk.w, walk.ti, e0, false);
+    wait_previous();
     float x[4], b[4] = {0.f, 0.f, 0.f, 0.f}, g[4];
     if (nx.vec) {
         load4(kFromGlobal ? p.x + nx.start + e0 : p.X + nx.base + e0, x);
@@ -219,8 +219,7 @@ cudaError_t launch_local_adamw(const Problem& p, const LaunchShape& ls, const Ad
     // the zero-state variants read less and use the grids of the state-reading ones
     const int grid = clamp_grid(from_x ? ls.grid_adamw_from_x : ls.grid_adamw, items);
     if (grid == 0) return cudaSuccess;
-    adamw_kernel_for(p.grad_bf16, from_x, zero_state)<<<grid, kThreads, 0, s>>>(p, a);
-    return cudaGetLastError();
+    return launch(adamw_kernel_for(p.grad_bf16, from_x, zero_state), grid, kThreads, 0, s, p.early, p, a);
 }
 
 cudaError_t launch_local_sgdm(const Problem& p, const LaunchShape& ls, const SgdmScalars& a, bool from_x,
@@ -228,8 +227,7 @@ cudaError_t launch_local_sgdm(const Problem& p, const LaunchShape& ls, const Sgd
     const uint64_t items = static_cast<uint64_t>(p.num_tiles) * p.n;
     const int grid = clamp_grid(from_x ? ls.grid_sgdm_from_x : ls.grid_sgdm, items);
     if (grid == 0) return cudaSuccess;
-    sgdm_kernel_for(p.grad_bf16, from_x, zero_state)<<<grid, kThreads, 0, s>>>(p, a);
-    return cudaGetLastError();
+    return launch(sgdm_kernel_for(p.grad_bf16, from_x, zero_state), grid, kThreads, 0, s, p.early, p, a);
 }
 
 }  // namespace dsm

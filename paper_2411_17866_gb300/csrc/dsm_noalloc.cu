@@ -234,6 +234,7 @@ extern "C" int dsm_global_step_noalloc(const dsm_layout* layout, uint32_t n, con
     g.philox_q0 = layout->first_element >> 2;
     uint32_t grid = 0;
     if ((err = launch_global(p, ls, g, s, &grid)) != cudaSuccess) return na_cuda(err, "launch global step");
+    p.early = true;  // (not the global step itself: the kernel before it writes the tile table)
     if ((err = launch_stats(p, grid, s)) != cudaSuccess) return na_cuda(err, "launch statistics");
     if (stats) {
         err = cudaMemcpyAsync(stats, p.stats, sizeof(TensorStats) * layout->count,

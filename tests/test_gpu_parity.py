@@ -208,6 +208,22 @@ def same_but_for_nan(got, want, what):
     assert_bitexact(got[~nan], want[~nan], what)
 
 
+@pytest.mark.parametrize("fused", [False, True], ids=["unfused", "fused"])
+@pytest.mark.parametrize("n", [3, 9])
+def test_captured_round_bitexact(n, fused):
+    """A round captured in a CUDA graph and replayed (its launches depend on one another programmatically)."""
+    hp = dataclasses.replace(ADAMW, flags=W.FLAG_FUSED_ROUND if fused else 0)
+    run, ora = dsm.DistributedSignMomentum(RAGGED, n, 2, hp), O.OracleRun(RAGGED, n, 2, hp)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        run.synthetic_round()
+    graph.replay()
+    ora.run_round()
+    compare_state(run, ora)
+    run.close()
+
+
 FUSED = [
     ("adamw-f32-n4-t3", ADAMW, 4, 3),
     ("adamw-bf16-n8-t2", dataclasses.replace(ADAMW, grad_dtype=W.BF16), 8, 2),
