@@ -190,10 +190,10 @@ __global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global
                 if (kGlobal == kGlobalRuntime) {
                     global_elem_rt<NW>(x[j], m[j], d, g, lam_g, ru[j], st);
                 } else if (kGlobal == kGlobalAdamW) {
-                    global_elem<NW, 4>(x[j], m[j], gv[j], d, NW, g, lam_g, ru[j], st);
+                    global_elem<NW, 4>(x[j], m[j], gv[j], d, g, lam_g, ru[j], st);
                 } else {
                     float unused = 0.f;
-                    global_elem<NW, 0>(x[j], m[j], unused, d, NW, g, lam_g, ru[j], st);
+                    global_elem<NW, 0>(x[j], m[j], unused, d, g, lam_g, ru[j], st);
                 }
             }
             store4(p.x + gi, x);
@@ -228,11 +228,11 @@ __global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global
                 global_elem_rt<NW>(x, m, d, g, lam_g, r, st);
             } else if (kGlobal == kGlobalAdamW) {
                 float v = p.gv[gj];
-                global_elem<NW, 4>(x, m, v, d, NW, g, lam_g, r, st);
+                global_elem<NW, 4>(x, m, v, d, g, lam_g, r, st);
                 p.gv[gj] = v;
             } else {
                 float unused = 0.f;
-                global_elem<NW, 0>(x, m, unused, d, NW, g, lam_g, r, st);
+                global_elem<NW, 0>(x, m, unused, d, g, lam_g, r, st);
             }
             p.x[gj] = x;
             p.m[gj] = m;

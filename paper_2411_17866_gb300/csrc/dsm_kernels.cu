@@ -166,126 +166,56 @@ __global__ void __launch_bounds__(kFillThreads) k_grad_fill(Problem p, GradKeys 
     }
 }
 
-// Global step on one element, any number of workers, reading each replica
-// once for the average and once more for the statistics.
+// Global step on one element of a partial group, more than 8 workers, by a warp:
+// lane l reads workers l and l + 32, and the sums take them in worker order by
+// shuffles.  (One thread reading one replica after the other made a tensor's
+// partial groups take longer than its tile: 20 us for 64 workers.)
 template <int MODE>
-__device__ __forceinline__ void global_elem_generic(const Problem& p, const GlobalScalars& g, float lam,
-                                                    uint64_t gi, ThreadStats& st) {
+__device__ __forceinline__ void global_elem_warp(const Problem& p, const GlobalScalars& g, float lam, uint64_t gi,
+                                                 ThreadStats& st) {
+    const uint32_t lane = threadIdx.x & 31u;
     float x = p.x[gi], m = p.m[gi], v = MODE == 4 ? p.gv[gi] : 0.f;
-    const float x0 = x;
+    float d[2] = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (lane + 32 * k < p.n) d[k] = __fsub_rn(x, p.X[(lane + 32 * k) * p.d_stride + gi]);
     float r = 0.f;
     if (MODE == 0 && g.sign_mode != 0)
         r = philox_unit(word_of(philox_block((gi >> 2) + g.philox_q0, g.philox_k0, g.philox_k1), gi & 3));
     float acc = 0.f;
-    for (uint32_t i = 0; i < p.n; ++i) acc = __fadd_rn(acc, __fsub_rn(x0, p.X[i * p.d_stride + gi]));
+#pragma unroll 1
+    for (uint32_t i = 0; i < p.n; ++i) acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, i < 32 ? d[0] : d[1], i & 31));
     const float D = __fdiv_rn(acc, g.n_f);
     float u, s;
     global_update<MODE>(D, x, m, v, g, lam, r, u, s);
-    const int sD = sgn(D);
-    float dr = 0.f;
     bool unan = true;
-    for (uint32_t i = 0; i < p.n; ++i) {
-        const float di = __fsub_rn(x0, p.X[i * p.d_stride + gi]);
-        const float ei = __fsub_rn(di, D);
-        dr = __fadd_rn(dr, __fmul_rn(ei, ei));
-        unan = unan && (sgn(di) == sD);
+    float sq[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float e = __fsub_rn(d[k], D);
+        sq[k] = __fmul_rn(e, e);
+        if (lane + 32 * k < p.n) unan = unan && sgn(d[k]) == sgn(D);
     }
-    csum_add(st.dsq, __fmul_rn(D, D));
-    csum_add(st.drift, dr);
-    st.zero += (s == 0.f);
-    st.flips += (sgn(u) != sD);
-    st.unanimous += unan;
-    st.clamped += (MODE == 0 && g.sign_mode != 0 && fabsf(u) > g.B);
-    p.x[gi] = x;
-    p.m[gi] = m;
-    if (MODE == 4) p.gv[gi] = v;
+    unan = __all_sync(0xffffffffu, unan);
+    float dr = 0.f;
+#pragma unroll 1
+    for (uint32_t i = 0; i < p.n; ++i) dr = __fadd_rn(dr, __shfl_sync(0xffffffffu, i < 32 ? sq[0] : sq[1], i & 31));
+    if (lane == 0) {
+        count_elem<MODE>(D, u, s, unan, g, st);
+        csum_add(st.drift, dr);
+        p.x[gi] = x;
+        p.m[gi] = m;
+        if (MODE == 4) p.gv[gi] = v;
+    }
     if (!g.skip_reset)
-        for (uint32_t i = 0; i < p.n; ++i) p.X[i * p.d_stride + gi] = x;
-}
-
-// Global step on a thread's 4 aligned elements for any number of workers:
-// 16-byte accesses, the replicas read once for the average and once more
-// (from L2) for the statistics, then overwritten by the reset.
-template <int MODE>
-__device__ __forceinline__ void global_vec_generic(const Problem& p, const GlobalScalars& g, float lam,
-                                                   uint64_t gi, ThreadStats& st) {
-    float x[4], m[4], v[4] = {0.f, 0.f, 0.f, 0.f}, acc[4] = {0.f, 0.f, 0.f, 0.f};
-    load4(p.x + gi, x);
-    load4(p.m + gi, m);
-    if (MODE == 4) load4(p.gv + gi, v);
-    // pass 1: the average; the loads of up to kGenChunk workers are issued before their additions,
-    // which stay in worker order (kept in L2 for pass 2)
-    constexpr uint32_t kGenChunk = 8;
-    for (uint32_t i0 = 0; i0 < p.n; i0 += kGenChunk) {
-        float4 r[kGenChunk];
 #pragma unroll
-        for (uint32_t c = 0; c < kGenChunk; ++c)
-            if (i0 + c < p.n) r[c] = *reinterpret_cast<const float4*>(p.X + (i0 + c) * p.d_stride + gi);
-#pragma unroll
-        for (uint32_t c = 0; c < kGenChunk; ++c) {
-            if (i0 + c < p.n) {
-                acc[0] = __fadd_rn(acc[0], __fsub_rn(x[0], r[c].x));
-                acc[1] = __fadd_rn(acc[1], __fsub_rn(x[1], r[c].y));
-                acc[2] = __fadd_rn(acc[2], __fsub_rn(x[2], r[c].z));
-                acc[3] = __fadd_rn(acc[3], __fsub_rn(x[3], r[c].w));
-            }
-        }
-    }
-    float ru[4] = {0.f, 0.f, 0.f, 0.f};
-    if (MODE == 0 && g.sign_mode != 0) {
-        const uint4 b = philox_block((gi >> 2) + g.philox_q0, g.philox_k0, g.philox_k1);
-        ru[0] = philox_unit(b.x); ru[1] = philox_unit(b.y); ru[2] = philox_unit(b.z); ru[3] = philox_unit(b.w);
-    }
-    float D[4], xn[4], dr[4] = {0.f, 0.f, 0.f, 0.f};
-    int sD[4];
-    bool unan[4] = {true, true, true, true};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        D[j] = __fdiv_rn(acc[j], g.n_f);
-        sD[j] = sgn(D[j]);
-        xn[j] = x[j];
-        float u, s;
-        global_update<MODE>(D[j], xn[j], m[j], v[j], g, lam, ru[j], u, s);
-        st.zero += (s == 0.f);
-        st.flips += (sgn(u) != sD[j]);
-        st.clamped += (MODE == 0 && g.sign_mode != 0 && fabsf(u) > g.B);
-        csum_add(st.dsq, __fmul_rn(D[j], D[j]));
-    }
-    // pass 2: the statistics and the reset, again kGenChunk workers' loads at a time
-    for (uint32_t i0 = 0; i0 < p.n; i0 += kGenChunk) {
-        float4 r[kGenChunk];
-#pragma unroll
-        for (uint32_t c = 0; c < kGenChunk; ++c)
-            if (i0 + c < p.n) r[c] = __ldcs(reinterpret_cast<const float4*>(p.X + (i0 + c) * p.d_stride + gi));
-#pragma unroll
-        for (uint32_t c = 0; c < kGenChunk; ++c) {
-            if (i0 + c < p.n) {
-                const float rr[4] = {r[c].x, r[c].y, r[c].z, r[c].w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float di = __fsub_rn(x[j], rr[j]);
-                    const float ei = __fsub_rn(di, D[j]);
-                    dr[j] = __fadd_rn(dr[j], __fmul_rn(ei, ei));
-                    unan[j] = unan[j] && (sgn(di) == sD[j]);
-                }
-                if (!g.skip_reset) store4(p.X + (i0 + c) * p.d_stride + gi, xn);
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        csum_add(st.drift, dr[j]);
-        st.unanimous += unan[j];
-    }
-    store4(p.x + gi, xn);
-    store4(p.m + gi, m);
-    if (MODE == 4) store4(p.gv + gi, v);
+        for (int k = 0; k < 2; ++k)
+            if (lane + 32 * k < p.n) p.X[(lane + 32 * k) * p.d_stride + gi] = x;
 }
 
 // K4: the fused global step (average over the replicas, sign-momentum update,
 // momentum update, reset of every replica unless g.skip_reset) with statistics.
-// NW > 0: exactly NW replicas, held in registers and double-buffered.
-// NW == 0: any n, one element at a time.
+// Exactly NW replicas (up to 8), held in registers and double-buffered.
 // Statistics: a CTA keeps per-thread sums while its successive tiles belong
 // to one tensor and reduces them only when the tensor changes (or at its last
 // tile), writing the segment's partial at the segment's last tile.  With a
@@ -294,12 +224,12 @@ __device__ __forceinline__ void global_vec_generic(const Problem& p, const Globa
 // min(G, tiles) tiles, which K5 sums.
 // CTAs per SM: what the double-buffered replicas leave room for (4 for n = 1, 3 up to n = 4, 2 above).
 template <int NW, int MODE>
-__global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_global(Problem p, GlobalScalars g) {
+__global__ void __launch_bounds__(kThreads, NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_global(Problem p, GlobalScalars g) {
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
-    constexpr int W = NW > 0 ? NW : 1;
+    constexpr int W = NW;
     uint32_t ti = blockIdx.x;
     TileDesc nt = p.tiles[ti];
-    bool nvec = NW > 0 && vector_ok(nt, e0);
+    bool nvec = vector_ok(nt, e0);
     wait_previous();
     float x[4], m[4], v[4] = {0.f, 0.f, 0.f, 0.f}, r[W][4];
     ThreadStats st;
@@ -325,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4
         const uint32_t next = ti + gridDim.x;
         if (next < p.num_tiles) {
             nt = p.tiles[next];
-            nvec = NW > 0 && vector_ok(nt, e0);
+            nvec = vector_ok(nt, e0);
             if (nvec) {
                 load4(p.x + nt.start + e0, x);
                 load4(p.m + nt.start + e0, m);
@@ -347,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4
                 float dif[W];
 #pragma unroll
                 for (int i = 0; i < W; ++i) dif[i] = __fsub_rn(cx[j], cr[i][j]);
-                global_elem<W, MODE>(cx[j], cm[j], cv[j], dif, W, g, lam, ru[j], st);
+                global_elem<W, MODE>(cx[j], cm[j], cv[j], dif, g, lam, ru[j], st);
             }
             store4(p.x + gi, cx);
             store4(p.m + gi, cm);
@@ -356,11 +286,128 @@ __global__ void __launch_bounds__(kThreads, NW == 0 || NW > 4 ? 2 : (NW == 1 ? 4
 #pragma unroll
                 for (int i = 0; i < W; ++i) store4(p.X + i * p.d_stride + gi, cx);
             }
-        } else if (NW == 0 && vector_ok(td, e0)) {
-            global_vec_generic<MODE>(p, g, lam, td.start + e0, st);
         }
-        if (uint32_t e; edge_element(td, e)) global_elem_generic<MODE>(p, g, lam, td.start + e, st);
+        if (uint32_t e; edge_element(td, e)) {
+            const uint64_t gj = td.start + e;
+            float xs = p.x[gj], ms = p.m[gj], vs = MODE == 4 ? p.gv[gj] : 0.f, dif[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) dif[i] = __fsub_rn(xs, p.X[i * p.d_stride + gj]);
+            float r = 0.f;
+            if (MODE == 0 && g.sign_mode != 0)
+                r = philox_unit(word_of(philox_block((gj >> 2) + g.philox_q0, g.philox_k0, g.philox_k1), gj & 3));
+            global_elem<W, MODE>(xs, ms, vs, dif, g, lam, r, st);
+            p.x[gj] = xs;
+            p.m[gj] = ms;
+            if (MODE == 4) p.gv[gj] = vs;
+            if (!g.skip_reset) {
+#pragma unroll
+                for (int i = 0; i < W; ++i) p.X[i * p.d_stride + gj] = xs;
+            }
+        }
         if (next >= p.num_tiles || nt.tensor != td.tensor) {  // uniform across the CTA
+            reduce_stats(st, p.partials + ti);
+            st = ThreadStats();
+        }
+    }
+}
+
+// K4 for more than 8 workers (up to NW): the replicas of a thread's E elements in registers, all of their loads in
+// flight at once, no second read for the statistics.  NW * E is 64: 4 elements a thread up to 16 workers, 2 up to 32,
+// 1 up to 64, a tile in 4 / E passes.  Bound by HBM bandwidth; 2 CTAs per SM hold 128 KB of loads in flight.  16
+// workers of 16 M parameters, reset deferred (1.28 GB): 223 us, against 330 us with 8 replicas at a time and a second
+// read from L2 for the statistics; 2 elements a thread in 4 CTAs per SM spill and are slower, in 3 the same.
+template <int NW, int E, int MODE>
+__global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalScalars g) {
+    uint32_t ti = blockIdx.x;
+    TileDesc nt = p.tiles[ti];
+    wait_previous();
+    ThreadStats st;
+    for (; ti < p.num_tiles; ti += gridDim.x) {
+        const TileDesc td = nt;
+        const uint32_t next = ti + gridDim.x;
+        if (next < p.num_tiles) nt = p.tiles[next];
+        const float lam = p.tensors[td.tensor].lam_global;
+#pragma unroll 1
+        for (uint32_t e = threadIdx.x * E; e < kTile && e < td.end(); e += kThreads * E) {
+            if (!vector_ok(td, e & ~3u)) continue;
+            const uint64_t gi = td.start + e;
+            float x[E], m[E], v[E], r[NW][E];
+            load_elems(p.x + gi, x);
+            // eight workers at a time, the last one again in the place of any beyond it, so that the loads are straight-
+            // line code: with a test of i for each, global AdamW for 64 workers waited for one load after the other
+            // (283 k parameters: 58 instead of 35 us)
+#pragma unroll
+            for (int i = 0; i < NW; i += 8) {
+                if (i < p.n) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) load_elems(p.X + min(i + k, int(p.n) - 1) * p.d_stride + gi, r[i + k]);
+                }
+            }
+            load_elems(p.m + gi, m);
+            if (MODE == 4) load_elems(p.gv + gi, v);
+            float ru[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) ru[j] = 0.f;
+            if (MODE == 0 && g.sign_mode != 0) {
+                const uint4 b = philox_block((gi >> 2) + g.philox_q0, g.philox_k0, g.philox_k1);
+#pragma unroll
+                for (int j = 0; j < E; ++j) ru[j] = philox_unit(word_of(b, (e + j) & 3u));
+            }
+            // the differences x - x_i, their sum in worker order, their extremes
+            float acc[E], lo[E], hi[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) { acc[j] = 0.f; lo[j] = INFINITY; hi[j] = -INFINITY; }
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                if (i < p.n) {
+#pragma unroll
+                    for (int j = 0; j < E; ++j) {
+                        r[i][j] = __fsub_rn(x[j], r[i][j]);
+                        acc[j] = __fadd_rn(acc[j], r[i][j]);
+                        lo[j] = fminf(lo[j], r[i][j]);
+                        hi[j] = fmaxf(hi[j], r[i][j]);
+                    }
+                }
+            }
+            float D[E], dr[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                D[j] = __fdiv_rn(acc[j], g.n_f);
+                float u, s;
+                global_update<MODE>(D[j], x[j], m[j], v[j], g, lam, ru[j], u, s);
+                // the signs of all differences are Delta's if Delta > 0 and the smallest is above 0, or Delta < 0 and
+                // the largest below 0 (none is NaN then: their sum would be), or Delta's sign is 0 and none is above
+                // or below 0; fminf and fmaxf pass over NaN, whose sign is 0
+                const bool unan =
+                    D[j] > 0.f ? lo[j] > 0.f : (D[j] < 0.f ? hi[j] < 0.f : !(hi[j] > 0.f) && !(lo[j] < 0.f));
+                count_elem<MODE>(D[j], u, s, unan, g, st);
+                dr[j] = 0.f;
+            }
+            store_elems(p.x + gi, x);
+            store_elems(p.m + gi, m);
+            if (MODE == 4) store_elems(p.gv + gi, v);
+            if (!g.skip_reset) {
+#pragma unroll
+                for (int i = 0; i < NW; ++i)
+                    if (i < p.n) store_elems(p.X + i * p.d_stride + gi, x);
+            }
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                if (i < p.n) {
+#pragma unroll
+                    for (int j = 0; j < E; ++j) {
+                        const float d = __fsub_rn(r[i][j], D[j]);
+                        dr[j] = __fadd_rn(dr[j], __fmul_rn(d, d));
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < E; ++j) csum_add(st.drift, dr[j]);
+        }
+        // the last warps first, as edge_element()
+        if (uint32_t e; edge_at(td, kThreads / 32 - 1 - threadIdx.x / 32, e))
+            global_elem_warp<MODE>(p, g, lam, td.start + e, st);
+        if (next >= p.num_tiles || nt.tensor != td.tensor) {  // uniform across the CTA (as in k_global)
             reduce_stats(st, p.partials + ti);
             st = ThreadStats();
         }
@@ -436,7 +483,8 @@ GlobalKernel global_kernel_mode(uint32_t n) {
         case 6: return k_global<6, MODE>;
         case 7: return k_global<7, MODE>;
         case 8: return k_global<8, MODE>;
-        default: return k_global<0, MODE>;
+        default: return n <= 16 ? k_global_many<16, 4, MODE>
+                                : (n <= 32 ? k_global_many<32, 2, MODE> : k_global_many<64, 1, MODE>);
     }
 }
 

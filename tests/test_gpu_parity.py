@@ -224,6 +224,24 @@ def test_captured_round_bitexact(n, fused):
     run.close()
 
 
+@pytest.mark.parametrize("mode", [W.GLOBAL_SIGN_MOMENTUM, W.GLOBAL_ADAMW], ids=["sign", "gadamw"])
+@pytest.mark.parametrize("n", [9, 15, 17, 24, 32, 33, 63, 64])
+def test_many_workers_bitexact(n, mode):
+    """The global step for more than 8 workers at the limits of its three forms (16, 32 and 64 workers), with tensors
+    whose partial groups a warp takes one element at a time, with the reset and with the reset deferred."""
+    tensors = _every_offset([1, 3, 6, 1030, 2048])
+    sign = W.RSIGN_PM if mode == W.GLOBAL_SIGN_MOMENTUM else W.SIGN
+    for flags in (0, W.FLAG_FUSED_ROUND):
+        hp = dataclasses.replace(SGDM, sign_mode=sign, global_mode=mode, flags=flags)
+        run, ora = dsm.DistributedSignMomentum(tensors, n, 1, hp), O.OracleRun(tensors, n, 1, hp, with_stats=True)
+        for _ in range(2):
+            stats = run.synthetic_round(with_stats=True)
+            ora.run_round()
+            compare_state(run, ora)
+            compare_stats(stats, ora.last_stats, n)
+        run.close()
+
+
 FUSED = [
     ("adamw-f32-n4-t3", ADAMW, 4, 3),
     ("adamw-bf16-n8-t2", dataclasses.replace(ADAMW, grad_dtype=W.BF16), 8, 2),
