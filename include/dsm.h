@@ -449,10 +449,8 @@ const char* dsm_last_error(void);
  * because every call rewrites the parts it reads.  Calls whose work
  * overlaps on the GPU (on different streams, or from different threads, on
  * the same device) race on the scratch array: order them on one stream or
- * serialise them.  The layout's tensor list is copied from host memory to
- * the device on the stream; from pageable host memory that copy has
- * consumed the list when the call returns, from pinned memory the list must
- * stay unchanged until the stream reaches it. */
+ * serialise them.  The layout's tensor list is consumed when the call
+ * returns. */
 #define DSM_NOALLOC_MAX_TENSORS 4096u
 #define DSM_NOALLOC_MAX_TILES   524288u
 #define DSM_NOALLOC_SCRATCH_BYTES 25657344u

@@ -108,8 +108,8 @@ struct Problem {
     float* opt_v;          // [n][d_stride] (AdamW only)
     void* grad;            // [n][d_stride], fp32 or bf16
     int grad_bf16;
-    bool early;            // kernels may start before the one before them has ended (wait_previous() in
-                           // dsm_device.cuh): the tables above are not written by a kernel just before
+    bool early;            // kernels may start before the one before them has ended: wait_previous() in dsm_device.cuh
+    bool fresh_tables;     // the kernel just before the global step writes the tables above
     StatPartial* partials; // [num_tiles]; only each CTA's last tile of a tensor is written
     TensorStats* stats;    // [num_tensors]
 };
@@ -160,6 +160,7 @@ struct LaunchShape {
 
 // Launchers (dsm_kernels.cu, dsm_local.cu, dsm_fused.cu).  Each returns the cudaError_t of its launch.
 cudaError_t query_launch_shape(const Problem& p, LaunchShape* out);
+cudaError_t query_global_shape(const Problem& p, LaunchShape* out);  // the global step's grid and sms only
 cudaError_t query_local_shape(const Problem& p, LaunchShape* out);  // the local steps' grids (dsm_local.cu)
 cudaError_t launch_init(const Problem& p, const LaunchShape& ls, uint64_t seed_key_init, int from_hash,
                         cudaStream_t s);

@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(kThreads, NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_gl
     const uint32_t e0 = threadIdx.x * kElemsPerThread;
     constexpr int W = NW;
     uint32_t ti = blockIdx.x;
+    if (p.fresh_tables) wait_previous();
     TileDesc nt = p.tiles[ti];
     bool nvec = vector_ok(nt, e0);
     wait_previous();
@@ -319,6 +320,7 @@ __global__ void __launch_bounds__(kThreads, NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_gl
 template <int NW, int E, int MODE>
 __global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalScalars g) {
     uint32_t ti = blockIdx.x;
+    if (p.fresh_tables) wait_previous();
     TileDesc nt = p.tiles[ti];
     wait_previous();
     ThreadStats st;
@@ -500,21 +502,26 @@ GlobalKernel global_kernel_for(uint32_t n, int mode) {
 
 }  // namespace
 
-cudaError_t query_launch_shape(const Problem& p, LaunchShape* out) {
+cudaError_t query_global_shape(const Problem& p, LaunchShape* out) {
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
-    int sms = 0;
-    err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    err = cudaDeviceGetAttribute(&out->sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    out->sms = sms;
+    out->grid_global = grid_for(global_kernel_for(p.n, p.global_mode), out->sms);
+    return cudaGetLastError();
+}
+
+cudaError_t query_launch_shape(const Problem& p, LaunchShape* out) {
+    const cudaError_t err = query_global_shape(p, out);
+    if (err != cudaSuccess) return err;
+    const int sms = out->sms;
     out->grid_init = grid_for(k_init, sms);
     out->grid_grad = p.grad_bf16 ? grid_for(k_grad_fill<true>, sms, 0, kFillThreads)
                                  : grid_for(k_grad_fill<false>, sms, 0, kFillThreads);
     cudaError_t e = query_local_shape(p, out);
     if (e != cudaSuccess) return e;
     if (fused_round_available(p) && (e = query_fused_shape(p, out)) != cudaSuccess) return e;
-    out->grid_global = grid_for(global_kernel_for(p.n, p.global_mode), sms);
     return cudaGetLastError();
 }
 

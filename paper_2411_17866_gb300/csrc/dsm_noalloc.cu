@@ -10,7 +10,7 @@
 #include <string>
 
 #include "dsm.h"
-#include "dsm_internal.h"
+#include "dsm_device.cuh"
 
 namespace dsm {
 namespace {
@@ -19,8 +19,8 @@ constexpr uint64_t align256(uint64_t v) { return (v + 255) / 256 * 256; }
 
 constexpr uint32_t kNaMaxTensors = DSM_NOALLOC_MAX_TENSORS;
 constexpr uint32_t kNaMaxTiles = DSM_NOALLOC_MAX_TILES;
-// Regions of the scratch array (byte offsets).
-constexpr uint64_t kOffLayout = 0;  // copy of the caller's dsm_tensor list
+// Regions of the scratch array (byte offsets); the first, 24 bytes a tensor, is not used.
+constexpr uint64_t kOffLayout = 0;
 constexpr uint64_t kOffTensors = align256(kOffLayout + sizeof(dsm_tensor) * kNaMaxTensors);
 constexpr uint64_t kOffTiles = align256(kOffTensors + sizeof(TensorDesc) * kNaMaxTensors);
 constexpr uint64_t kOffPartials = align256(kOffTiles + sizeof(TileDesc) * uint64_t(kNaMaxTiles));
@@ -31,68 +31,75 @@ static_assert(kScratchBytes == DSM_NOALLOC_SCRATCH_BYTES, "scratch size in dsm.h
 // The scratch array: shared by every call on a device, kept until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-// One CTA: tensor offsets and tile ranges by a prefix sum over the tensor list.
-__global__ void __launch_bounds__(kThreads) k_noalloc_tensor_table(unsigned char* scratch, uint32_t count,
-                                                                   float lam_global) {
-    const dsm_tensor* in = reinterpret_cast<const dsm_tensor*>(scratch + kOffLayout);
-    TensorDesc* out = reinterpret_cast<TensorDesc*>(scratch + kOffTensors);
-    __shared__ unsigned long long s_el[kThreads], s_ti[kThreads];
-    const uint32_t per = (count + kThreads - 1) / kThreads;
-    const uint32_t b = threadIdx.x * per, e = min(b + per, count);
-    unsigned long long el = 0, ti = 0;
-    for (uint32_t i = b; i < e; ++i) {
-        el += in[i].numel;
-        ti += (in[i].numel + kTile - 1) / kTile;
-    }
-    s_el[threadIdx.x] = el;
-    s_ti[threadIdx.x] = ti;
+// Up to kListTensors consecutive tensors, passed to the kernel by value: where each starts (elements, tiles), with
+// the end of the last, and whether weight decay applies.  The host, which checks the list anyway, adds up the sizes.
+constexpr uint32_t kListTensors = 256;
+struct TensorList {
+    uint32_t first, count;                // tensors first .. first + count - 1
+    float lam_global;
+    uint32_t wd[kListTensors / 32];       // bit i: tensor first + i
+    uint32_t tile[kListTensors + 1];
+    uint64_t off[kListTensors + 1];
+};
+
+// The tensor and tile tables of the listed tensors: tile ti belongs to the last tensor whose first tile is <= ti.
+// One launch for up to 256 tensors, with no copy before it.  (The list copied from the host, a prefix sum over it by
+// one CTA and the tile table in a second kernel took 16 us of the 50 us of a call on 3.4 M parameters.)
+__global__ void __launch_bounds__(kThreads) k_noalloc_tables(unsigned char* scratch, const __grid_constant__ TensorList l) {
+    TensorDesc* tensors = reinterpret_cast<TensorDesc*>(scratch + kOffTensors);
+    TileDesc* tiles = reinterpret_cast<TileDesc*>(scratch + kOffTiles);
+    __shared__ uint32_t s_tile[kListTensors + 1];
+    for (uint32_t i = threadIdx.x; i <= l.count; i += kThreads) s_tile[i] = l.tile[i];
     __syncthreads();
-    if (threadIdx.x == 0) {  // exclusive scan of the 256 chunk sums
-        unsigned long long a = 0, c = 0;
-        for (uint32_t k = 0; k < kThreads; ++k) {
-            const unsigned long long va = s_el[k], vc = s_ti[k];
-            s_el[k] = a;
-            s_ti[k] = c;
-            a += va;
-            c += vc;
+    wait_previous();  // the previous call's kernels read the tables
+    const uint32_t id = blockIdx.x * kThreads + threadIdx.x, threads = gridDim.x * kThreads;
+    for (uint32_t i = id; i < l.count; i += threads) {
+        TensorDesc t{};
+        t.off = l.off[i];
+        t.numel = l.off[i + 1] - l.off[i];
+        t.lam_global = (l.wd[i / 32] >> (i % 32) & 1u) ? l.lam_global : 0.0f;
+        t.tile_begin = s_tile[i];
+        t.tile_end = s_tile[i + 1];
+        tensors[l.first + i] = t;
+    }
+    for (uint32_t ti = s_tile[0] + id; ti < s_tile[l.count]; ti += threads) {
+        uint32_t lo = 0, hi = l.count;  // first tensor with a first tile beyond ti
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) / 2;
+            if (s_tile[mid] <= ti) lo = mid + 1;
+            else hi = mid;
         }
-    }
-    __syncthreads();
-    el = s_el[threadIdx.x];
-    ti = s_ti[threadIdx.x];
-    for (uint32_t i = b; i < e; ++i) {
-        TensorDesc t;
-        t.off = el;
-        t.numel = in[i].numel;
-        t.scale = in[i].grad_scale;
-        t.scale2 = 0.0f;
-        t.lam_local = 0.0f;
-        t.lam_global = in[i].wd ? lam_global : 0.0f;
-        t.kind = in[i].kind;
-        t.tile_begin = static_cast<uint32_t>(ti);
-        ti += (in[i].numel + kTile - 1) / kTile;
-        t.tile_end = static_cast<uint32_t>(ti);
-        t.pad = 0;
-        out[i] = t;
-        el += in[i].numel;
+        const uint32_t i = lo - 1;
+        tiles[ti] = make_tile(l.off[i], l.off[i + 1] - l.off[i], l.first + i, ti - s_tile[i]);
     }
 }
 
-// Tile table: tile ti belongs to the last tensor whose tile_begin <= ti.
-__global__ void __launch_bounds__(kThreads) k_noalloc_tile_table(unsigned char* scratch, uint32_t count,
-                                                                 uint32_t num_tiles) {
-    const TensorDesc* t = reinterpret_cast<const TensorDesc*>(scratch + kOffTensors);
-    TileDesc* tiles = reinterpret_cast<TileDesc*>(scratch + kOffTiles);
-    for (uint32_t ti = blockIdx.x * blockDim.x + threadIdx.x; ti < num_tiles; ti += gridDim.x * blockDim.x) {
-        uint32_t lo = 0, hi = count;  // first tensor with tile_begin > ti
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) / 2;
-            if (t[mid].tile_begin <= ti) lo = mid + 1;
-            else hi = mid;
+// Launches k_noalloc_tables for every kListTensors tensors of the layout.
+cudaError_t launch_tables(unsigned char* scratch, const dsm_layout* layout, float lam_global, cudaStream_t s) {
+    uint64_t off = 0;
+    uint32_t tile = 0;
+    for (uint32_t first = 0; first < layout->count; first += kListTensors) {
+        TensorList l{};
+        l.first = first;
+        l.count = layout->count - first < kListTensors ? layout->count - first : kListTensors;
+        l.lam_global = lam_global;
+        for (uint32_t i = 0; i < l.count; ++i) {
+            const dsm_tensor& t = layout->tensors[first + i];
+            l.off[i] = off;
+            l.tile[i] = tile;
+            if (t.wd) l.wd[i / 32] |= 1u << (i % 32);
+            off += t.numel;
+            tile += static_cast<uint32_t>((t.numel + kTile - 1) / kTile);
         }
-        const TensorDesc& T = t[lo - 1];
-        tiles[ti] = make_tile(T.off, T.numel, lo - 1, ti - T.tile_begin);
+        l.off[l.count] = off;
+        l.tile[l.count] = tile;
+        const uint32_t work = l.tile[l.count] - l.tile[0] > l.count ? l.tile[l.count] - l.tile[0] : l.count;
+        const uint32_t blocks = (work + kThreads - 1) / kThreads;
+        const cudaError_t err = launch(k_noalloc_tables, static_cast<int>(blocks < 1024 ? blocks : 1024), kThreads, 0, s,
+                                       true, scratch, l);
+        if (err != cudaSuccess) return err;
     }
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -191,32 +198,28 @@ extern "C" int dsm_global_step_noalloc(const dsm_layout* layout, uint32_t n, con
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
     // Tensor and tile tables, rebuilt in the scratch array by every call.
-    err = cudaMemcpyAsync(scratch + kOffLayout, layout->tensors, sizeof(dsm_tensor) * layout->count,
-                          cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return na_cuda(err, "copy the tensor list");
-    k_noalloc_tensor_table<<<1, kThreads, 0, s>>>(scratch, layout->count, hp->g_wd);
-    if ((err = cudaGetLastError()) != cudaSuccess) return na_cuda(err, "launch tensor table");
-    const uint32_t num_tiles = static_cast<uint32_t>(tiles);
-    const uint32_t tb = (num_tiles + kThreads - 1) / kThreads;
-    k_noalloc_tile_table<<<tb < 1024 ? tb : 1024, kThreads, 0, s>>>(scratch, layout->count, num_tiles);
-    if ((err = cudaGetLastError()) != cudaSuccess) return na_cuda(err, "launch tile table");
+    if ((err = launch_tables(scratch, layout, hp->g_wd, s)) != cudaSuccess) return na_cuda(err, "launch the tables");
 
     Problem p{};
     p.tensors = reinterpret_cast<const TensorDesc*>(scratch + kOffTensors);
     p.tiles = reinterpret_cast<const TileDesc*>(scratch + kOffTiles);
     p.num_tensors = layout->count;
-    p.num_tiles = num_tiles;
+    p.num_tiles = static_cast<uint32_t>(tiles);
     p.n = n;
     p.d_stride = replica_stride;
     p.x = x;
     p.m = m;
     p.X = replicas;
     p.partials = reinterpret_cast<StatPartial*>(scratch + kOffPartials);
-    p.stats = reinterpret_cast<TensorStats*>(scratch + kOffStats);
+    // statistics in device memory are written there at once
+    const bool in_place = stats && stats_is_device && reinterpret_cast<uintptr_t>(stats) % alignof(TensorStats) == 0;
+    p.stats = in_place ? reinterpret_cast<TensorStats*>(stats) : reinterpret_cast<TensorStats*>(scratch + kOffStats);
 
     p.global_mode = hp->global_mode;
+    p.early = true;
+    p.fresh_tables = true;
     LaunchShape ls;
-    if ((err = query_launch_shape(p, &ls)) != cudaSuccess) return na_cuda(err, "occupancy query");
+    if ((err = query_global_shape(p, &ls)) != cudaSuccess) return na_cuda(err, "occupancy query");
     GlobalScalars g{};
     g.b1 = hp->g_b1;
     g.b2 = hp->g_b2;
@@ -234,9 +237,8 @@ extern "C" int dsm_global_step_noalloc(const dsm_layout* layout, uint32_t n, con
     g.philox_q0 = layout->first_element >> 2;
     uint32_t grid = 0;
     if ((err = launch_global(p, ls, g, s, &grid)) != cudaSuccess) return na_cuda(err, "launch global step");
-    p.early = true;  // (not the global step itself: the kernel before it writes the tile table)
     if ((err = launch_stats(p, grid, s)) != cudaSuccess) return na_cuda(err, "launch statistics");
-    if (stats) {
+    if (stats && !in_place) {
         err = cudaMemcpyAsync(stats, p.stats, sizeof(TensorStats) * layout->count,
                               stats_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
         if (err != cudaSuccess) return na_cuda(err, "copy statistics");

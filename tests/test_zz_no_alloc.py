@@ -218,6 +218,30 @@ def test_noalloc_checks_every_buffer_and_the_tensor_list():
     assert e.value.code == dsm.DSM_EINVAL and "reserved" in str(e.value)
 
 
+@pytest.mark.parametrize("count", [255, 256, 257, 600])
+def test_noalloc_many_tensors(count):
+    """Lists of more tensors than one launch of the table kernel takes, empty ones and the last tile of a launch among
+    them, against the handle path."""
+    _need_gpu()
+    rng = np.random.default_rng(count)
+    sizes = rng.choice([0, 1, 2, 5, 64, 1023, 1024, 1025, 3001], count)
+    sizes[-1] = 7
+    tensors = tuple(W.Tensor(f"t{i}", int(k), W.KIND_WEIGHT, 1e-3, wd=int(i % 3 != 0)) for i, k in enumerate(sizes))
+    n, hp = 3, W.HParams()
+    run = dsm.DistributedSignMomentum(tensors, n, 1, hp)
+    run.fill_synthetic_grads(0)
+    run.local_step()
+    x, m, reps = _caller_buffers(run, n)
+    info = run.info()
+    dev_stats = torch.zeros(count * 6, dtype=torch.float64, device="cuda")
+    _noalloc(tensors, n, hp, info.gamma, info.round, x, m, reps, run.d_stride, dev_stats, stats_is_device=True)
+    want = run.global_step(with_stats=True)
+    torch.cuda.synchronize()
+    _assert_same_as_handle(run, n, x, m, reps)
+    _stats_close(_device_stats_rows(dev_stats, count), want, n)
+    run.close()
+
+
 def dsm_max_tiles():
     return 524288
 
