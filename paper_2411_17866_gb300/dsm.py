@@ -127,14 +127,29 @@ def _check(rc: int, func: str) -> None:
         raise DsmError(rc, func, last_error())
 
 
-def _stream(stream) -> c_void_p:
+_current_stream = None
+
+
+def _make_current_stream():
+    """A function that returns the cudaStream_t of torch's current stream as an int.  The raw handle costs 0.3 us;
+    torch.cuda.current_stream() builds a Stream object on every call (3.2 of the 6.0 us of a local_step() call)."""
+    import torch
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
+
+
+def _stream(stream) -> int:
     """A cudaStream_t from a torch stream, an int handle, or None (torch's current stream)."""
+    global _current_stream
     if stream is None:
-        import torch
-        return c_void_p(torch.cuda.current_stream().cuda_stream)
+        if _current_stream is None:
+            _current_stream = _make_current_stream()
+        return _current_stream()
     if isinstance(stream, int):
-        return c_void_p(stream)
-    return c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def make_layout(tensors, first_element: int = 0):
