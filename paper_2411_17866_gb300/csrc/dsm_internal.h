@@ -178,7 +178,7 @@ constexpr int kFusedZeroState = 2;  // the base-optimizer states are zero: none 
 constexpr int kFusedDropState = 4;  // the new base-optimizer states are not written (the round resets them)
 bool fused_round_available(const Problem& p);
 cudaError_t query_fused_shape(const Problem& p, LaunchShape* out);  // sets grid_fused (out->sms must be set)
-// The global-step launchers write per-tile statistics partials and set *grid to the number of CTAs
+// The global-step launchers write per-tile statistics partials and set *grid to the number of CTAs (or clusters)
 // they launched; launch_stats reduces those partials per tensor and needs that grid.
 cudaError_t launch_fused_last_global(const Problem& p, const LaunchShape& ls, const AdamScalars& a,
                                      const SgdmScalars& sa, const GlobalScalars& g, int opts, cudaStream_t s,

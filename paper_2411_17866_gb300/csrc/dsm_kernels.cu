@@ -21,6 +21,8 @@
 // never contracts into FMAs, so each result is the fp32 value of the
 // paper's expression evaluated one operation at a time.
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -312,25 +314,46 @@ __global__ void __launch_bounds__(kThreads, NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_gl
     }
 }
 
+// reduce_stats() over the CTAs of a cluster: each one's sums in its shared memory, added in rank order by the first.
+__device__ __forceinline__ void reduce_stats_cluster(const ThreadStats& st, StatPartial* out) {
+    __shared__ StatPartial s_part;
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    reduce_stats(st, &s_part);
+    cluster.sync();
+    if (cluster.block_rank() == 0 && threadIdx.x == 0) {
+        StatPartial o = s_part;
+        for (uint32_t r = 1; r < cluster.num_blocks(); ++r) {
+            const StatPartial q = *cluster.map_shared_rank(&s_part, r);
+            o.delta_sq += q.delta_sq; o.drift += q.drift;
+            o.zero_sign += q.zero_sign; o.flips += q.flips; o.unanimous += q.unanimous; o.clamped += q.clamped;
+        }
+        *out = o;
+    }
+    cluster.sync();  // no CTA ends, or writes its sums again, before they are read
+}
+
 // K4 for more than 8 workers (up to NW): the replicas of a thread's E elements in registers, all of their loads in
 // flight at once, no second read for the statistics.  NW * E is 64: 4 elements a thread up to 16 workers, 2 up to 32,
-// 1 up to 64, a tile in 4 / E passes.  Bound by HBM bandwidth; 2 CTAs per SM hold 128 KB of loads in flight.  16
+// 1 up to 64, a tile by a cluster of 4 / E CTAs that add up their statistics through distributed shared memory, or by
+// one CTA in as many passes.  Bound by HBM bandwidth; 2 CTAs per SM hold 128 KB of loads in flight.  16
 // workers of 16 M parameters, reset deferred (1.28 GB): 223 us, against 330 us with 8 replicas at a time and a second
 // read from L2 for the statistics; 2 elements a thread in 4 CTAs per SM spill and are slower, in 3 the same.
-template <int NW, int E, int MODE>
+template <int NW, int E, int MODE, bool kCluster>
 __global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalScalars g) {
-    uint32_t ti = blockIdx.x;
+    constexpr uint32_t parts = kCluster ? 4 / E : 1;
+    const uint32_t part = blockIdx.x % parts, clusters = gridDim.x / parts;
+    uint32_t ti = blockIdx.x / parts;
     if (p.fresh_tables) wait_previous();
     TileDesc nt = p.tiles[ti];
     wait_previous();
     ThreadStats st;
-    for (; ti < p.num_tiles; ti += gridDim.x) {
+    for (; ti < p.num_tiles; ti += clusters) {
         const TileDesc td = nt;
-        const uint32_t next = ti + gridDim.x;
+        const uint32_t next = ti + clusters;
         if (next < p.num_tiles) nt = p.tiles[next];
         const float lam = p.tensors[td.tensor].lam_global;
 #pragma unroll 1
-        for (uint32_t e = threadIdx.x * E; e < kTile && e < td.end(); e += kThreads * E) {
+        for (uint32_t e = (part * kThreads + threadIdx.x) * E; e < kTile && e < td.end(); e += parts * kThreads * E) {
             if (!vector_ok(td, e & ~3u)) continue;
             const uint64_t gi = td.start + e;
             float x[E], m[E], v[E], r[NW][E];
@@ -406,11 +429,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalSc
 #pragma unroll
             for (int j = 0; j < E; ++j) csum_add(st.drift, dr[j]);
         }
-        // the last warps first, as edge_element()
-        if (uint32_t e; edge_at(td, kThreads / 32 - 1 - threadIdx.x / 32, e))
-            global_elem_warp<MODE>(p, g, lam, td.start + e, st);
-        if (next >= p.num_tiles || nt.tensor != td.tensor) {  // uniform across the CTA (as in k_global)
-            reduce_stats(st, p.partials + ti);
+        // the last warps of the last CTA first, as edge_element()
+        if (uint32_t ee; part == parts - 1 && edge_at(td, kThreads / 32 - 1 - threadIdx.x / 32, ee))
+            global_elem_warp<MODE>(p, g, lam, td.start + ee, st);
+        if (next >= p.num_tiles || nt.tensor != td.tensor) {  // uniform across the cluster (as in k_global)
+            if (kCluster) reduce_stats_cluster(st, p.partials + ti);
+            else reduce_stats(st, p.partials + ti);
             st = ThreadStats();
         }
     }
@@ -475,7 +499,7 @@ __global__ void __launch_bounds__(kThreads) k_stats(Problem p, uint32_t producer
 using GlobalKernel = void (*)(Problem, GlobalScalars);
 
 template <int MODE>
-GlobalKernel global_kernel_mode(uint32_t n) {
+GlobalKernel global_kernel_mode(uint32_t n, bool cluster) {
     switch (n) {
         case 1: return k_global<1, MODE>;
         case 2: return k_global<2, MODE>;
@@ -485,18 +509,20 @@ GlobalKernel global_kernel_mode(uint32_t n) {
         case 6: return k_global<6, MODE>;
         case 7: return k_global<7, MODE>;
         case 8: return k_global<8, MODE>;
-        default: return n <= 16 ? k_global_many<16, 4, MODE>
-                                : (n <= 32 ? k_global_many<32, 2, MODE> : k_global_many<64, 1, MODE>);
+        default: break;
     }
+    if (n <= 16) return k_global_many<16, 4, MODE, false>;
+    if (n <= 32) return cluster ? k_global_many<32, 2, MODE, true> : k_global_many<32, 2, MODE, false>;
+    return cluster ? k_global_many<64, 1, MODE, true> : k_global_many<64, 1, MODE, false>;
 }
 
-GlobalKernel global_kernel_for(uint32_t n, int mode) {
+GlobalKernel global_kernel_for(uint32_t n, int mode, bool cluster) {
     switch (mode) {
-        case 1: return global_kernel_mode<1>(n);
-        case 2: return global_kernel_mode<2>(n);
-        case 3: return global_kernel_mode<3>(n);
-        case 4: return global_kernel_mode<4>(n);
-        default: return global_kernel_mode<0>(n);
+        case 1: return global_kernel_mode<1>(n, cluster);
+        case 2: return global_kernel_mode<2>(n, cluster);
+        case 3: return global_kernel_mode<3>(n, cluster);
+        case 4: return global_kernel_mode<4>(n, cluster);
+        default: return global_kernel_mode<0>(n, cluster);
     }
 }
 
@@ -508,7 +534,7 @@ cudaError_t query_global_shape(const Problem& p, LaunchShape* out) {
     if (err != cudaSuccess) return err;
     err = cudaDeviceGetAttribute(&out->sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    out->grid_global = grid_for(global_kernel_for(p.n, p.global_mode), out->sms);
+    out->grid_global = grid_for(global_kernel_for(p.n, p.global_mode, false), out->sms);
     return cudaGetLastError();
 }
 
@@ -537,12 +563,23 @@ cudaError_t launch_grad_fill(const Problem& p, const LaunchShape& ls, const Grad
     return launch(p.grad_bf16 ? k_grad_fill<true> : k_grad_fill<false>, grid, kFillThreads, 0, s, p.early, p, k);
 }
 
+// CTAs that share a tile in the global step for more than 8 workers: a cluster of 4 / E (see k_global_many) as long as
+// every tile's then runs at the same time; beyond that one CTA takes a tile in 4 / E passes, which leaves no CTA
+// waiting for another's sums.  Rounds of one SGD-momentum step, 64 workers, one CTA / clusters: 3 k parameters 20.8 /
+// 12.1 us, 30 k 23.5 / 14.9, 200 k (784 CTAs) 61.9 / 59.4, 283 k 85.2 / 90.8, 4 M 1100 / 1151.
+static uint32_t tile_ctas(const Problem& p, const LaunchShape& ls) {
+    const uint32_t parts = p.n <= 16 ? 1 : (p.n <= 32 ? 2 : 4);
+    return uint64_t(p.num_tiles) * parts <= static_cast<uint64_t>(ls.grid_global) ? parts : 1;
+}
+
 cudaError_t launch_global(const Problem& p, const LaunchShape& ls, const GlobalScalars& g, cudaStream_t s,
                           uint32_t* grid_used) {
-    const int grid = clamp_grid(ls.grid_global, p.num_tiles);
-    *grid_used = static_cast<uint32_t>(grid);
-    if (grid == 0) return cudaSuccess;
-    return launch(global_kernel_for(p.n, p.global_mode), grid, kThreads, 0, s, p.early, p, g);
+    const uint32_t parts = tile_ctas(p, ls);
+    const int tiles = clamp_grid(ls.grid_global, p.num_tiles);  // (clusters of) CTAs
+    *grid_used = static_cast<uint32_t>(tiles);
+    if (tiles == 0) return cudaSuccess;
+    return launch_clusters(global_kernel_for(p.n, p.global_mode, parts > 1), tiles * static_cast<int>(parts), parts,
+                           kThreads, 0, s, p.early, p, g);
 }
 
 cudaError_t launch_stats(const Problem& p, uint32_t producer_grid, cudaStream_t s) {
