@@ -62,12 +62,16 @@ __host__ __device__ constexpr size_t fused_smem(bool adamw, bool bf16, int nw, i
             size_t(fused_glob_sets(adamw, nw)) * fused_globals(global) * 16) * kThreads;
 }
 
-// CTAs per SM: 4 up to n = 4 and 3 above, as many as the staging allows.  Left to itself the compiler gave the
-// global AdamW instantiations 111-212 registers for n > 4, 2 CTAs or 1: K6 for n = 6, bf16 gradients, 16.3 M
-// parameters took 436 us against 390 us with 3.
+// CTAs per SM: 4 up to n = 4 and 3 above, as many as the staging allows; the global AdamW step, which needs more
+// registers, 3 up to n = 6 and 2 above.  (Rounds of two steps on 16.3 M parameters, us.  Left to itself the compiler took
+// 111-212 registers for global AdamW with n > 4; n = 4, bf16 gradients: 4 CTAs 531, 3 516; n = 8: 3 CTAs 1004, 2 949.)
+__host__ __device__ constexpr int fused_ctas(int nw, int global) {
+    return global == kGlobalAdamW ? (nw <= 6 ? 3 : 2) : (nw <= 4 ? 4 : 3);
+}
+
 template <bool kAdamW, bool kBf16, int NW, int kGlobal>
-__global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global(Problem p, AdamScalars a, SgdmScalars sa,
-                                                                GlobalScalars g, int opts) {
+__global__ void __launch_bounds__(kThreads, fused_ctas(NW, kGlobal))
+    k_fused_last_global(Problem p, AdamScalars a, SgdmScalars sa, GlobalScalars g, int opts) {
     constexpr int kFusedDepth = fused_depth(kAdamW, NW);
     constexpr int kStates = fused_states(kAdamW), kGlobals = fused_globals(kGlobal);
     constexpr int kGradBytes = kBf16 ? 8 : 16;
@@ -204,13 +208,15 @@ __global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global
 #pragma unroll
             for (int w = 0; w < NW; ++w, ++it) issue(next_issue++);
         }
-        if (uint32_t e; edge_element(td, e)) {
+        // a partial group's element by a warp, the last warps first (as edge_element()): lane w runs worker w's step,
+        // all workers' loads at the same time (one thread, worker after worker, took 8 us for n = 8)
+        if (uint32_t e; edge_at(td, kThreads / 32 - 1 - threadIdx.x / 32, e)) {
             const uint64_t gj = td.start + e;
-            float x = p.x[gj], m = p.m[gj], d[NW];
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                const uint64_t o = w * p.d_stride + gj;
-                float xi = from_global ? x : p.X[o], mi = zero_state ? 0.f : p.opt_m[o];
+            const uint32_t lane = threadIdx.x & 31u;
+            float xe = p.x[gj], me = p.m[gj], ve = kGlobal == kGlobalAdamW ? p.gv[gj] : 0.f, dw = 0.f, d[NW];
+            if (lane < NW) {
+                const uint64_t o = lane * p.d_stride + gj;
+                float xi = from_global ? xe : p.X[o], mi = zero_state ? 0.f : p.opt_m[o];
                 if (kAdamW) {
                     float vi = zero_state ? 0.f : p.opt_v[o];
                     adamw_elem(xi, mi, vi, load_grad1(p.grad, kBf16, o), a, lam_l);
@@ -219,23 +225,20 @@ __global__ void __launch_bounds__(kThreads, NW <= 4 ? 4 : 3) k_fused_last_global
                     sgdm_elem(xi, mi, load_grad1(p.grad, kBf16, o), sa);
                 }
                 if (keep_state) p.opt_m[o] = mi;
-                d[w] = __fsub_rn(x, xi);
+                dw = __fsub_rn(xe, xi);
             }
+#pragma unroll
+            for (int w = 0; w < NW; ++w) d[w] = __shfl_sync(0xffffffffu, dw, w);
             float r = 0.f;
             if (kGlobal == kGlobalSign && g.sign_mode != 0)
                 r = philox_unit(word_of(philox_block((gj >> 2) + g.philox_q0, g.philox_k0, g.philox_k1), gj & 3));
-            if (kGlobal == kGlobalRuntime) {
-                global_elem_rt<NW>(x, m, d, g, lam_g, r, st);
-            } else if (kGlobal == kGlobalAdamW) {
-                float v = p.gv[gj];
-                global_elem<NW, 4>(x, m, v, d, g, lam_g, r, st);
-                p.gv[gj] = v;
-            } else {
-                float unused = 0.f;
-                global_elem<NW, 0>(x, m, unused, d, g, lam_g, r, st);
+            if (lane == 0) {
+                if (kGlobal == kGlobalRuntime) global_elem_rt<NW>(xe, me, d, g, lam_g, r, st);
+                else global_elem<NW, kGlobal == kGlobalAdamW ? 4 : 0>(xe, me, ve, d, g, lam_g, r, st);
+                p.x[gj] = xe;
+                p.m[gj] = me;
+                if (kGlobal == kGlobalAdamW) p.gv[gj] = ve;
             }
-            p.x[gj] = x;
-            p.m[gj] = m;
         }
         const uint32_t next = ti + gridDim.x;
         if (next >= p.num_tiles || p.tiles[next].tensor != td.tensor) {  // uniform across the CTA
