@@ -298,7 +298,7 @@ int dsm_local_step(dsm_handle* h, dsm_stream_t stream);
  * and their transfer overlapped with the update.  src is a dense [n][d]
  * array of the gradient type in host memory, the caller's; pinned memory
  * makes the copies asynchronous (pageable memory works, without overlap).
- * The model is cut into chunks of whole tiles (about 64 MB of gradients
+ * The model is cut into chunks of whole tiles (about 16 MB of gradients
  * each, at most 64): for every chunk the call enqueues the copy of its n
  * gradient slices on copy_stream and, on stream, the local step on that
  * chunk once its copy has landed, so that the copy of one chunk runs while
@@ -306,9 +306,10 @@ int dsm_local_step(dsm_handle* h, dsm_stream_t stream);
  * enqueued on stream before the call; work enqueued on stream after the
  * call follows every copy and every update.  copy_stream may equal stream
  * (no overlap).  Same results, bit for bit, as dsm_load_grads followed by
- * dsm_local_step; with the fused round's last step the copies are enqueued
- * and the update is left to dsm_global_step, as for dsm_local_step.  The
- * first call creates the handle's chunk events (cudaEventCreate); the
+ * dsm_local_step; where the copies overlap nothing (one chunk, or
+ * copy_stream equal to stream) the fused round's last step only enqueues
+ * them and leaves the update to dsm_global_step, as dsm_local_step does.
+ * The first call creates the handle's chunk events (cudaEventCreate); the
  * environment variable DSM_HOST_GRAD_CHUNK_BYTES, read then, sets another
  * chunk size.  src must stay unchanged until the copies have completed (until
  * stream reaches work enqueued after the call).
