@@ -503,7 +503,7 @@ int dsm_create(const dsm_layout* layout, uint32_t n, uint32_t tau, const dsm_hpa
         delete h;
         return cuda_fail(e, what);
     };
-    if ((err = query_launch_shape(p, &h->shape)) != cudaSuccess) return bail(err, "occupancy query");
+    if ((err = query_launch_shape(p, h->tensors.data(), &h->shape)) != cudaSuccess) return bail(err, "occupancy query");
     h->fused = (hp->flags & DSM_FLAG_FUSED_ROUND) && fused_round_available(p);
     h->lazy_reset = (hp->flags & DSM_FLAG_FUSED_ROUND) != 0;
     // The tables are copied from the handle's own vectors, which outlive the copies.

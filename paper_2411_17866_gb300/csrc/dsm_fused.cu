@@ -1,6 +1,8 @@
 // Host side of the fused round (DSM_FLAG_FUSED_ROUND): which kernel, how much
 // shared memory, the launch.  The kernel is in dsm_fused.cuh.
 
+#include <algorithm>
+
 #include "dsm_fused.cuh"
 
 namespace dsm {
@@ -29,13 +31,26 @@ bool fused_round_available(const Problem& p) {
     return p.global_mode >= 0 && p.global_mode <= 4 && p.n >= 1 && p.n <= kMaxUnrolledWorkers;
 }
 
-cudaError_t query_fused_shape(const Problem& p, LaunchShape* out) {
+cudaError_t query_fused_shape(const Problem& p, const TensorDesc* tensors, LaunchShape* out) {
     if (!fused_round_available(p)) return cudaSuccess;
     const FusedKernel fk = fused_kernel_for(p, p.opt_v != nullptr);
     const size_t smem = fused_smem_for(p, p.opt_v != nullptr);
     cudaError_t e = cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     out->grid_fused = grid_for(fk, out->sms, smem);
+    // AdamW with 2 to 4 workers on more than L2 holds streams better with 2 CTAs per SM (rounds of two steps, us, 2 / 3
+    // CTAs: 184 M parameters, fp32, n = 2 3152 / 3256, n = 3 4434 / 4558, n = 4 5769 / 5862, slower with any number in
+    // between; n = 4, 1.6 M 49.3 / 46.6, 1.9 M 63.7 / 61.4, 2.2 M 76.0 / 76.0, 3 M 102 / 104; n = 2, 3 M 49.1 / 46.8,
+    // 3.7 M 67.7 / 69.0).  Not so n = 1, n >= 5, SGD-momentum and the global AdamW step.
+    // Nor where more than a third of the tiles end a CTA's run of one tensor, each with a reduction of its statistics
+    // that the other CTAs of the SM run on through (29.8 M in 174 tensors, n = 4, bf16 gradients: 933 / 915).
+    const uint64_t bytes = p.d_stride * (uint64_t(p.n) * (12 + (p.grad_bf16 ? 2 : 4)) + 8);
+    if (p.opt_v && p.n >= 2 && p.n <= 4 && p.global_mode != 4 && bytes > 150000000ull) {
+        const uint32_t two = 2 * static_cast<uint32_t>(out->sms);
+        uint64_t runs = 0;
+        for (uint32_t t = 0; t < p.num_tensors; ++t) runs += std::min(tensors[t].tile_end - tensors[t].tile_begin, two);
+        if (3 * runs <= p.num_tiles) out->grid_fused = std::min(out->grid_fused, static_cast<int>(two));
+    }
     return cudaSuccess;
 }
 

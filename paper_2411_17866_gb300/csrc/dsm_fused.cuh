@@ -62,12 +62,12 @@ __host__ __device__ constexpr size_t fused_smem(bool adamw, bool bf16, int nw, i
             size_t(fused_glob_sets(adamw, nw)) * fused_globals(global) * 16) * kThreads;
 }
 
-// CTAs per SM: 4 up to n = 4 and 3 above, as many as the staging allows; the global AdamW step, which needs more
-// registers, 3 up to n = 6 and 2 above.  (Rounds of two steps on 16.3 M parameters, us.  Left to itself the compiler took
-// 111-212 registers for global AdamW with n > 4; n = 4, bf16 gradients: 4 CTAs 531, 3 516; n = 8: 3 CTAs 1004, 2 949.)
-__host__ __device__ constexpr int fused_ctas(int nw, int global) {
-    return global == kGlobalAdamW ? (nw <= 6 ? 3 : 2) : (nw <= 4 ? 4 : 3);
-}
+// CTAs per SM that the registers are for: 3; 2 for the global AdamW step, which needs more of them, from n = 7 on.
+// (Rounds of two steps, us.  4 CTAs of 64 registers for n <= 4: GPT-2 S, SGD-momentum, n = 2 1534 against 1477, n = 4
+// 2886 against 2806; in L2, 1 M parameters, AdamW, n = 4 30.6 against 29.2.  Global AdamW, 16.3 M parameters, bf16
+// gradients, n = 8: 3 CTAs 1004, 2 949; left to itself the compiler took 111-212 registers for n > 4.)  See
+// query_fused_shape() for the CTAs that are launched.
+__host__ __device__ constexpr int fused_ctas(int nw, int global) { return global == kGlobalAdamW && nw > 6 ? 2 : 3; }
 
 template <bool kAdamW, bool kBf16, int NW, int kGlobal>
 __global__ void __launch_bounds__(kThreads, fused_ctas(NW, kGlobal))

@@ -159,7 +159,8 @@ struct LaunchShape {
 };
 
 // Launchers (dsm_kernels.cu, dsm_local.cu, dsm_fused.cu).  Each returns the cudaError_t of its launch.
-cudaError_t query_launch_shape(const Problem& p, LaunchShape* out);
+// `tensors`: the tensor table in host memory.
+cudaError_t query_launch_shape(const Problem& p, const TensorDesc* tensors, LaunchShape* out);
 cudaError_t query_global_shape(const Problem& p, LaunchShape* out);  // the global step's grid and sms only
 cudaError_t query_local_shape(const Problem& p, LaunchShape* out);  // the local steps' grids (dsm_local.cu)
 cudaError_t launch_init(const Problem& p, const LaunchShape& ls, uint64_t seed_key_init, int from_hash,
@@ -177,7 +178,7 @@ constexpr int kFusedFromX = 1;      // the replicas' reset is pending: every wor
 constexpr int kFusedZeroState = 2;  // the base-optimizer states are zero: none is read
 constexpr int kFusedDropState = 4;  // the new base-optimizer states are not written (the round resets them)
 bool fused_round_available(const Problem& p);
-cudaError_t query_fused_shape(const Problem& p, LaunchShape* out);  // sets grid_fused (out->sms must be set)
+cudaError_t query_fused_shape(const Problem& p, const TensorDesc* tensors, LaunchShape* out);  // sets grid_fused (out->sms must be set)
 // The global-step launchers write per-tile statistics partials and set *grid to the number of CTAs (or clusters)
 // they launched; launch_stats reduces those partials per tensor and needs that grid.
 cudaError_t launch_fused_last_global(const Problem& p, const LaunchShape& ls, const AdamScalars& a,

@@ -400,12 +400,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalSc
                 D[j] = __fdiv_rn(acc[j], g.n_f);
                 float u, s;
                 global_update<MODE>(D[j], x[j], m[j], v[j], g, lam, ru[j], u, s);
-                // the signs of all differences are Delta's if Delta > 0 and the smallest is above 0, or Delta < 0 and
-                // the largest below 0 (none is NaN then: their sum would be), or Delta's sign is 0 and none is above
-                // or below 0; fminf and fmaxf pass over NaN, whose sign is 0
-                const bool unan =
-                    D[j] > 0.f ? lo[j] > 0.f : (D[j] < 0.f ? hi[j] < 0.f : !(hi[j] > 0.f) && !(lo[j] < 0.f));
-                count_elem<MODE>(D[j], u, s, unan, g, st);
+                count_elem<MODE>(D[j], u, s, same_signs(D[j], lo[j], hi[j]), g, st);
                 dr[j] = 0.f;
             }
             store_elems(p.x + gi, x);
@@ -538,7 +533,7 @@ cudaError_t query_global_shape(const Problem& p, LaunchShape* out) {
     return cudaGetLastError();
 }
 
-cudaError_t query_launch_shape(const Problem& p, LaunchShape* out) {
+cudaError_t query_launch_shape(const Problem& p, const TensorDesc* tensors, LaunchShape* out) {
     const cudaError_t err = query_global_shape(p, out);
     if (err != cudaSuccess) return err;
     const int sms = out->sms;
@@ -547,7 +542,7 @@ cudaError_t query_launch_shape(const Problem& p, LaunchShape* out) {
                                  : grid_for(k_grad_fill<false>, sms, 0, kFillThreads);
     cudaError_t e = query_local_shape(p, out);
     if (e != cudaSuccess) return e;
-    if (fused_round_available(p) && (e = query_fused_shape(p, out)) != cudaSuccess) return e;
+    if (fused_round_available(p) && (e = query_fused_shape(p, tensors, out)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

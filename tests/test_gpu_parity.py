@@ -201,6 +201,35 @@ def test_adamw_over_the_whole_range_bitexact(n, hp):
         run.close()
 
 
+@pytest.mark.parametrize("mode", [W.GLOBAL_SIGN_MOMENTUM, W.GLOBAL_ADAMW], ids=["sign", "gadamw"])
+@pytest.mark.parametrize("n,fused", [(3, False), (4, False), (3, True), (7, True), (8, True), (11, False), (20, False)])
+def test_global_step_over_the_whole_range_bitexact(n, fused, mode):
+    """Worker models of every magnitude around x = 0 (the local step leaves them as they are: no gradient, no momentum):
+    the average's and the global AdamW's branch-free divisions inside and outside their ranges."""
+    d = 1 << 14
+    rng = np.random.default_rng(n)
+    hp = dataclasses.replace(SGDM, mu=0.0, sign_mode=W.SIGN, global_mode=mode, flags=W.FLAG_FUSED_ROUND if fused else 0)
+    tensors, x0 = (W.Tensor("t", d, W.KIND_WEIGHT, 1e-3),), np.zeros(d, np.float32)
+    run = dsm.DistributedSignMomentum(tensors, n, 1, hp, x0=torch.from_numpy(x0))
+    ora = O.OracleRun(tensors, n, 1, hp, x0=x0)
+    exps = np.repeat(rng.integers(-149, 126, d // 4), 4) + rng.integers(-2, 3, d)   # groups of 4 of similar size
+    for i in range(n):
+        v = (rng.uniform(1, 2, d) * 2.0 ** exps * rng.choice([-1.0, 1.0], d)).astype(np.float32)
+        v[rng.random(d) < 0.02] = 0.0
+        run.write(dsm.BUF_REPLICA, torch.from_numpy(v), worker=i)
+        ora.X[i][:] = v
+    run.local_step()
+    with np.errstate(all="ignore"):
+        ora.local_step([np.zeros(d, np.float32)] * n)
+        run.global_step()
+        ora.global_step()
+    for which, want, what in ((dsm.BUF_X, ora.x, "x"), (dsm.BUF_M, ora.m, "m")):
+        same_but_for_nan(run.read(which).numpy(), want, what)
+    if mode == W.GLOBAL_ADAMW:
+        same_but_for_nan(run.read(dsm.BUF_GLOBAL_V).numpy(), ora.gv, "global v")
+    run.close()
+
+
 def same_but_for_nan(got, want, what):
     got, want = np.asarray(got), np.asarray(want, np.float32)
     nan = np.isnan(want)
