@@ -468,7 +468,7 @@ int dsm_create(const dsm_layout* layout, uint32_t n, uint32_t tau, const dsm_hpa
         const uint64_t count = (t.numel + kTile - 1) / kTile;
         for (uint64_t c = 0; c < count; ++c) h->tiles.push_back(make_tile(off, t.numel, i, c));
         td.tile_end = static_cast<uint32_t>(h->tiles.size());
-        td.pad = 0;
+        td.ticket = 0;
         off += t.numel;
     }
 

@@ -312,6 +312,7 @@ __global__ void __launch_bounds__(kThreads, NW > 4 ? 2 : (NW == 1 ? 4 : 3)) k_gl
             st = ThreadStats();
         }
     }
+    if (p.sum_stats) sum_stats(p, gridDim.x);
 }
 
 // reduce_stats() over the CTAs of a cluster: each one's sums in its shared memory, added in rank order by the first.
@@ -433,6 +434,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalSc
             st = ThreadStats();
         }
     }
+    if (p.sum_stats) sum_stats(p, clusters);
 }
 
 // K5: per-tensor statistics from the tile partials, in a fixed order: a
@@ -573,12 +575,14 @@ cudaError_t launch_global(const Problem& p, const LaunchShape& ls, const GlobalS
     const int tiles = clamp_grid(ls.grid_global, p.num_tiles);  // (clusters of) CTAs
     *grid_used = static_cast<uint32_t>(tiles);
     if (tiles == 0) return cudaSuccess;
+    Problem q = p;
+    q.sum_stats = stats_in_kernel(p);
     return launch_clusters(global_kernel_for(p.n, p.global_mode, parts > 1), tiles * static_cast<int>(parts), parts,
-                           kThreads, 0, s, p.early, p, g);
+                           kThreads, 0, s, p.early, q, g);
 }
 
 cudaError_t launch_stats(const Problem& p, uint32_t producer_grid, cudaStream_t s) {
-    if (p.num_tensors == 0) return cudaSuccess;
+    if (p.num_tensors == 0 || stats_in_kernel(p)) return cudaSuccess;
     return launch(k_stats, static_cast<int>(p.num_tensors), kThreads, 0, s, p.early, p, producer_grid);
 }
 

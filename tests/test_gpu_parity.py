@@ -271,6 +271,23 @@ def test_many_workers_bitexact(n, mode):
         run.close()
 
 
+@pytest.mark.parametrize("fused", [False, True], ids=["unfused", "fused"])
+@pytest.mark.parametrize("sizes", [(5,), (1024, 3, 0, 6000), (7000, 1000)], ids=["1-tile", "8-tiles", "9-tiles"])
+@pytest.mark.parametrize("n", [1, 4, 9, 40])
+def test_statistics_of_tiny_models(n, sizes, fused):
+    """Up to 8 tiles the global step's own kernel sums the statistics; several rounds on one handle (the CTAs' ticket
+    starts again), more CTAs than tensors and clusters among them."""
+    tensors = tuple(W.Tensor(f"t{i}", k, W.KIND_WEIGHT, 1e-2) for i, k in enumerate(sizes))
+    hp = dataclasses.replace(ADAMW, flags=W.FLAG_FUSED_ROUND if fused else 0)
+    run, ora = dsm.DistributedSignMomentum(tensors, n, 1, hp), O.OracleRun(tensors, n, 1, hp, with_stats=True)
+    for _ in range(3):
+        stats = run.synthetic_round(with_stats=True)
+        ora.run_round()
+        compare_stats(stats, ora.last_stats, n)
+    compare_state(run, ora)
+    run.close()
+
+
 FUSED = [
     ("adamw-f32-n4-t3", ADAMW, 4, 3),
     ("adamw-bf16-n8-t2", dataclasses.replace(ADAMW, grad_dtype=W.BF16), 8, 2),
