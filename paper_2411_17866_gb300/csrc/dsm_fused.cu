@@ -62,9 +62,7 @@ cudaError_t launch_fused_last_global(const Problem& p, const LaunchShape& ls, co
     *grid_used = static_cast<uint32_t>(grid);
     if (grid == 0) return cudaSuccess;
     const bool adamw = p.opt_v != nullptr;
-    Problem q = p;
-    q.sum_stats = stats_in_kernel(p);
-    return launch(fused_kernel_for(p, adamw), grid, kThreads, fused_smem_for(p, adamw), s, p.early, q, a, sa, g, opts);
+    return launch(fused_kernel_for(p, adamw), grid, kThreads, fused_smem_for(p, adamw), s, p.early, p, a, sa, g, opts);
 }
 
 }  // namespace dsm

@@ -246,7 +246,6 @@ __global__ void __launch_bounds__(kThreads, fused_ctas(NW, kGlobal))
             st = ThreadStats();
         }
     }
-    if (p.sum_stats) sum_stats(p, gridDim.x);
     cp_async_wait<0>();  // the groups issued past the last tile are empty; nothing is left in flight
 }
 

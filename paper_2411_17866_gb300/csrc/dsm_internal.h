@@ -109,7 +109,7 @@ struct Problem {
     void* grad;            // [n][d_stride], fp32 or bf16
     int grad_bf16;
     bool early;            // kernels may start before the one before them has ended: wait_previous() in dsm_device.cuh
-    bool sum_stats;        // the global step's kernel sums the statistics itself (stats_in_kernel())
+    bool sum_stats;        // the global step's kernel (K4) sums the statistics itself
     bool fresh_tables;     // the kernel just before the global step writes the tables above
     StatPartial* partials; // [num_tiles]; only each CTA's last tile of a tensor is written
     TensorStats* stats;    // [num_tensors]
@@ -181,19 +181,14 @@ constexpr int kFusedDropState = 4;  // the new base-optimizer states are not wri
 bool fused_round_available(const Problem& p);
 cudaError_t query_fused_shape(const Problem& p, const TensorDesc* tensors, LaunchShape* out);  // sets grid_fused (out->sms must be set)
 // The global-step launchers write per-tile statistics partials and set *grid to the number of CTAs (or clusters)
-// they launched; launch_stats reduces those partials per tensor and needs that grid.
+// they launched, or to 0 if the kernel sums the statistics itself; launch_stats reduces those partials per tensor
+// and needs that grid.
 cudaError_t launch_fused_last_global(const Problem& p, const LaunchShape& ls, const AdamScalars& a,
                                      const SgdmScalars& sa, const GlobalScalars& g, int opts, cudaStream_t s,
                                      uint32_t* grid);
 cudaError_t launch_global(const Problem& p, const LaunchShape& ls, const GlobalScalars& g, cudaStream_t s,
                           uint32_t* grid);
 cudaError_t launch_stats(const Problem& p, uint32_t producer_grid, cudaStream_t s);
-
-// Whether the kernel that produces the statistics' partials also sums them (the last of its CTAs does), without K5: a
-// launch less for models so small that a round is its launches, up to 8 tiles (rounds of one SGD-momentum step, n = 4,
-// without / with K5: 4.5 k parameters in 6 tensors 6.8 / 7.7 us; 30 tiles 8.1 / 7.6, 244 tiles 14.4 / 10.1).
-constexpr uint32_t kSumStatsTiles = 8;
-inline bool stats_in_kernel(const Problem& p) { return p.num_tiles <= kSumStatsTiles && p.num_tensors <= 4 * kSumStatsTiles; }
 
 // Sets the calling thread's message returned by dsm_last_error() (dsm_api.cpp).
 void set_last_error_message(const char* msg);
