@@ -19,7 +19,8 @@
 // All method arithmetic uses the explicit round-to-nearest intrinsics
 // (__fadd_rn, __fmul_rn, __fdiv_rn, __fsqrt_rn, ...), which the compiler
 // never contracts into FMAs, so each result is the fp32 value of the
-// paper's expression evaluated one operation at a time.
+// paper's expression evaluated one operation at a time (AdamW's divisions use
+// fused multiply-adds for the same correctly rounded quotients).
 
 #include <cooperative_groups.h>
 
