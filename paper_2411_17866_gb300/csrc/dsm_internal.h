@@ -157,6 +157,7 @@ struct LaunchShape {
     int sms = 0;
     int grid_grad = 0, grid_adamw = 0, grid_sgdm = 0, grid_global = 0, grid_init = 0;
     int grid_fused = 0, grid_adamw_from_x = 0, grid_sgdm_from_x = 0;
+    int grid_adamw_zero = 0, grid_adamw_zero_from_x = 0;  // the AdamW step that reads no state
 };
 
 // Launchers (dsm_kernels.cu, dsm_local.cu, dsm_fused.cu).  Each returns the cudaError_t of its launch.

@@ -177,7 +177,10 @@ cudaError_t query_local_shape(const Problem& p, LaunchShape* out) {
                                            : grid_for(k_local_adamw<false, false, false>, sms), adamw_ctas);
     // The SGD-momentum step fits 6 CTAs per SM, but 4 stream better (GB300, GPT-2 L layout, n = 8:
     // 0.96 of the copy bandwidth with 4, 0.91 with 6, 0.91 with 3), as many as the AdamW step holds.
-    constexpr int kSgdmCtasPerSm = 4;
+    // From x, which the n workers of a tile read once from HBM, 5 do (GPT-2 S, n = 4, fp32, rounds of two steps, us: 4 / 4.5
+    // / 5 / 6 CTAs per SM 2800 / 2720 / 2703 / 2812; n = 8 5115 / 5036 / 4978 / 5244; 16 M, n = 16, one step 847 / 825 /
+    // 814 / 848).
+    constexpr int kSgdmCtasPerSm = 4, kSgdmCtasPerSmFromX = 5;
     out->grid_sgdm = std::min(p.grad_bf16 ? grid_for(k_local_sgdm<true, false, false>, sms)
                                           : grid_for(k_local_sgdm<false, false, false>, sms), kSgdmCtasPerSm * sms);
     {  // the from-x variants (first local step after a lazy reset)
@@ -186,8 +189,16 @@ cudaError_t query_local_shape(const Problem& p, LaunchShape* out) {
                                           adamw_ctas_from_x);
         out->grid_sgdm_from_x = std::min(p.grad_bf16 ? grid_for(k_local_sgdm<true, true, false>, sms)
                                                      : grid_for(k_local_sgdm<false, true, false>, sms),
-                                         kSgdmCtasPerSm * sms);
+                                         kSgdmCtasPerSmFromX * sms);
     }
+    // The AdamW step that reads no state (the first of a round that restarts the optimizer) has fewer bytes in flight per
+    // thread.  From x (GPT-2 S, n = 4, fp32, rounds of two steps, us) 3.5 / 4.5 / 5 CTAs per SM 2868 / 2764 / 2799; 16.3
+    // M, n = 6, bf16 4 / 4.5 / 5 565 / 556 / 547; from the replicas (n = 4, fp32) 3 / 4 / 5 4542 / 4478 / 4585.
+    out->grid_adamw_zero_from_x =
+        std::min(p.grad_bf16 ? grid_for(k_local_adamw<true, true, true>, sms)
+                             : grid_for(k_local_adamw<false, true, true>, sms), p.grad_bf16 ? 5 * sms : 9 * sms / 2);
+    out->grid_adamw_zero = std::min(p.grad_bf16 ? grid_for(k_local_adamw<true, false, true>, sms)
+                                                : grid_for(k_local_adamw<false, false, true>, sms), 4 * sms);
     return cudaGetLastError();
 }
 
@@ -216,8 +227,9 @@ static SgdmKernel sgdm_kernel_for(bool bf16, bool from_x, bool zero_state) {
 cudaError_t launch_local_adamw(const Problem& p, const LaunchShape& ls, const AdamScalars& a, bool from_x,
                                bool zero_state, cudaStream_t s) {
     const uint64_t items = static_cast<uint64_t>(p.num_tiles) * p.n;
-    // the zero-state variants read less and use the grids of the state-reading ones
-    const int grid = clamp_grid(from_x ? ls.grid_adamw_from_x : ls.grid_adamw, items);
+    const int most = zero_state ? (from_x ? ls.grid_adamw_zero_from_x : ls.grid_adamw_zero)
+                                : (from_x ? ls.grid_adamw_from_x : ls.grid_adamw);
+    const int grid = clamp_grid(most, items);
     if (grid == 0) return cudaSuccess;
     return launch(adamw_kernel_for(p.grad_bf16, from_x, zero_state), grid, kThreads, 0, s, p.early, p, a);
 }
