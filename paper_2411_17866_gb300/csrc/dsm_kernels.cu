@@ -3,18 +3,19 @@
 // synthetic gradients (K1), the global step (K4) and its statistics (K5).
 // The local steps are in dsm_local.cu, the fused round in dsm_fused.cuh.
 //
-// Every kernel is a persistent, grid-stride loop over work items: tiles of
-// at most kTile = 1024 elements that lie inside one tensor (for the local
-// steps, a tile of one worker).  A CTA of 256 threads takes one item at a
-// time; each thread owns 4 consecutive elements and moves them with one
-// 16-byte load or store per fp32 stream (8 bytes per bf16 stream), so every
-// warp instruction covers 512 contiguous bytes.  (K1 instead runs 64-thread
-// CTAs whose threads own four such groups of a tile.)  The local and global
-// steps double-buffer in registers: a thread issues the loads of its next
-// item before it computes the current one, so the HBM requests of one item
-// are in flight during the arithmetic of the previous one.  The work is streaming and
-// elementwise, bound by HBM bandwidth; nothing is a contraction, and no tensor
-// core is used.
+// Every kernel is a grid-stride loop over work items, persistent but for K1
+// (whose grid has more CTAs than are resident): tiles of at most kTile = 1024
+// elements that lie inside one tensor (for the local steps, a tile of one
+// worker).  A CTA of 256 threads takes one item at a time; each thread owns 4
+// consecutive elements and moves them with one 16-byte load or store per fp32
+// stream (8 bytes per bf16 stream), so every warp instruction covers 512
+// contiguous bytes.  (K1 instead runs 64-thread CTAs whose threads own four
+// such groups of a tile.)  The local and global steps double-buffer in
+// registers: a thread issues the loads of its next item before it computes the
+// current one, so the HBM requests of one item are in flight during the
+// arithmetic of the previous one.  The work is streaming and elementwise,
+// bound by HBM bandwidth (K1: by instruction issue); nothing is a contraction,
+// and no tensor core is used.
 //
 // All method arithmetic uses the explicit round-to-nearest intrinsics
 // (__fadd_rn, __fmul_rn, __fdiv_rn, __fsqrt_rn, ...), which the compiler
@@ -541,8 +542,13 @@ cudaError_t query_launch_shape(const Problem& p, const TensorDesc* tensors, Laun
     if (err != cudaSuccess) return err;
     const int sms = out->sms;
     out->grid_init = grid_for(k_init, sms);
-    out->grid_grad = p.grad_bf16 ? grid_for(k_grad_fill<true>, sms, 0, kFillThreads)
-                                 : grid_for(k_grad_fill<false>, sms, 0, kFillThreads);
+    // K1 runs up to 300 CTAs per SM, of which 20 are resident: bound by
+    // instruction issue, it gains when a CTA's end makes room for the next
+    // (us a fill, 20 / 80 / 300 CTAs per SM / one CTA a tile: GPT-2 S, n = 4,
+    // fp32 339 / 328 / 325 / 325; n = 1 141.6 / 135.6 / 134.1 / 135.2; GPT-2 M,
+    // n = 4, bf16 1018 / 979 / 970 / 969; 1 M, n = 4 4.9 for 20 as for 300).
+    constexpr int kFillCtasPerSm = 300;
+    out->grid_grad = kFillCtasPerSm * sms;
     cudaError_t e = query_local_shape(p, out);
     if (e != cudaSuccess) return e;
     if (fused_round_available(p) && (e = query_fused_shape(p, tensors, out)) != cudaSuccess) return e;
