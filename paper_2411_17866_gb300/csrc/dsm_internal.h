@@ -110,7 +110,7 @@ struct Problem {
     int grad_bf16;
     bool early;            // kernels may start before the one before them has ended: wait_previous() in dsm_device.cuh
     bool sum_stats;        // the global step's kernel (K4) sums the statistics itself
-    bool fresh_tables;     // the kernel just before the global step writes the tables above
+    bool fresh_tables;     // a kernel of the same call writes the tables above: K4 and K5 wait before they read them
     StatPartial* partials; // [num_tiles]; only each CTA's last tile of a tensor is written
     TensorStats* stats;    // [num_tensors]
 };

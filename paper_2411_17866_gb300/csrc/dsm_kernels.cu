@@ -444,6 +444,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_global_many(Problem p, GlobalSc
 // G CTAs (see K4).
 __global__ void __launch_bounds__(kThreads) k_stats(Problem p, uint32_t producer_grid) {
     const uint32_t T = blockIdx.x;
+    if (p.fresh_tables) wait_previous();
     const TensorDesc td = p.tensors[T];
     wait_previous();
     double a = 0.0, b = 0.0;

@@ -242,6 +242,57 @@ def test_noalloc_many_tensors(count):
     run.close()
 
 
+@pytest.mark.parametrize("n", [2, 9])
+def test_noalloc_back_to_back_calls_on_two_layouts(n):
+    """Calls on one stream with nothing between them: few tiles in hundreds of tensors, then other tile ranges under the
+    same tensor numbers.  Each call's statistics use its own tables."""
+    _need_gpu()
+    hp, rng = W.HParams(), np.random.default_rng(n)
+    layouts = [tuple(W.Tensor(f"s{i}", int(k), W.KIND_WEIGHT, 1e-3) for i, k in enumerate(rng.integers(0, 40, 200))),
+               tuple(W.Tensor(f"l{i}", int(k), W.KIND_WEIGHT, 1e-3) for i, k in enumerate(rng.integers(1, 20000, 150)))]
+    bufs, outs = [], []
+    for tensors in layouts:
+        d = sum(t.numel for t in tensors)
+        stride = -(-d // 64) * 64
+        g = torch.Generator("cuda").manual_seed(d)
+        x = torch.randn(d, device="cuda", generator=g)
+        reps = x.repeat(n, 1) + 1e-3 * torch.randn(n, d, device="cuda", generator=g)
+        flat = torch.zeros(n, stride, device="cuda")
+        flat[:, :d] = reps
+        bufs.append((tensors, x, flat, stride))
+    calls = 8
+    for c in range(calls):
+        tensors, x, flat, stride = bufs[c % 2]
+        outs.append((x.clone(), torch.zeros_like(x), flat.clone(),
+                     torch.full((len(tensors), 6), -1.0, dtype=torch.float64, device="cuda")))
+    layout, chp = [dsm.make_layout(b[0]) for b in bufs], dsm.make_hparams(hp)
+    torch.cuda.synchronize()
+    for c in range(calls):
+        x, m, flat, stats = outs[c]
+        dsm.dsm_global_step_noalloc(layout[c % 2], n, chp, 1e-3, 0, x.data_ptr(), m.data_ptr(), flat.data_ptr(),
+                                    bufs[c % 2][3], stats.data_ptr(), stats_is_device=True)
+    torch.cuda.synchronize()
+    for c in range(calls):
+        tensors, x, flat, stride = bufs[c % 2]
+        got = _device_stats_rows(outs[c][3], len(tensors))
+        d = x.numel()
+        dif = (x[None] - flat[:, :d]).cpu().numpy()
+        acc = np.zeros(d, np.float32)
+        for i in range(n):
+            acc = acc + dif[i]
+        delta = acc / np.float32(n)
+        unanimous = (np.sign(dif) == np.sign(delta)).all(0)
+        off = 0
+        for T, t in enumerate(tensors):
+            part = slice(off, off + t.numel)
+            off += t.numel
+            want = float((delta[part].astype(np.float64) ** 2).sum())
+            assert abs(got[T]["delta_sq"] - want) <= stats_rtol(n) * want, (c, T)
+            assert got[T]["unanimous"] == int(unanimous[part].sum()), (c, T)
+    for c in range(2, calls):
+        assert torch.equal(outs[c][0], outs[c % 2][0]) and torch.equal(outs[c][3], outs[c % 2][3]), c
+
+
 def dsm_max_tiles():
     return 524288
 
