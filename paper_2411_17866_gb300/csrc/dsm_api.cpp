@@ -283,17 +283,7 @@ void next_local_scalars(const dsm_handle* h, AdamScalars* a, SgdmScalars* sa, do
     if (h->hp.base == DSM_BASE_ADAMW) {
         *nb1 = h->b1_pow * double(h->hp.b1);
         *nb2 = h->b2_pow * double(h->hp.b2);
-        a->b1 = h->hp.b1;
-        a->omb1 = float(1.0 - double(h->hp.b1));
-        a->b2 = h->hp.b2;
-        a->omb2 = float(1.0 - double(h->hp.b2));
-        a->bc1 = float(1.0 - *nb1);
-        a->bc2 = float(1.0 - *nb2);
-        a->lr = h->gamma;
-        a->eps = h->hp.eps;
-        a->rbc1 = float(1.0 / double(a->bc1));
-        a->rbc2 = float(1.0 / double(a->bc2));
-        a->newton = a->bc1 >= 0x1p-24f && a->bc2 >= 0x1p-24f && a->eps <= 0x1p60f;
+        *a = make_adam_scalars(h->hp.b1, h->hp.b2, h->hp.eps, h->gamma, *nb1, *nb2);
     } else {
         sa->mu = h->hp.mu;
         sa->lr = h->gamma;

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kThreads, fused_ctas(NW, kGlobal))
                     take(reinterpret_cast<const float4*>(grad_slot(it)), gr);
                 }
                 const uint64_t o = w * p.d_stride + gi;
-                if (kAdamW) adamw_group(xi, mi, vi, gr, a, lam_l);
+                if (kAdamW) adamw_group<NW >= 5 && kGlobal != kGlobalAdamW>(xi, mi, vi, gr, a, lam_l);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     if (!kAdamW) sgdm_elem(xi[j], mi[j], gr[j], sa);

@@ -115,6 +115,11 @@ struct Problem {
     TensorStats* stats;    // [num_tensors]
 };
 
+constexpr int kNewton = 1;        // adamw_group()'s, on moments in the usual ranges
+constexpr int kNewtonSparse = 2;  // adamw_rest()'s, which take zeros as well
+constexpr int kNewtonLowM = 4;    // and a denormal m (bc1 = 1)
+constexpr int kNewtonLowV = 8;    // and a denormal v (bc2 = 1)
+
 // Scalars of one AdamW local step (all fp32, computed once on the host).
 struct AdamScalars {
     float b1, omb1;        // beta1, 1 - beta1
@@ -122,8 +127,30 @@ struct AdamScalars {
     float bc1, bc2;        // 1 - beta1^j, 1 - beta2^j
     float lr, eps;
     float rbc1, rbc2;      // 1/bc1 and 1/bc2, correctly rounded
-    int newton;            // the scalars lie in the ranges that adamw_group() needs for its Newton forms
+    int newton;            // kNewton* bits: the Newton forms (adamw_group(), adamw_rest()) that the scalars allow
+    float mhi, vhi;        // the largest |m| and v that adamw_rest()'s take
 };
+
+// The scalars of the step whose beta powers are p1 = beta1^j and p2 = beta2^j.
+inline AdamScalars make_adam_scalars(float b1, float b2, float eps, float lr, double p1, double p2) {
+    AdamScalars a{};
+    a.b1 = b1;
+    a.omb1 = float(1.0 - double(b1));
+    a.b2 = b2;
+    a.omb2 = float(1.0 - double(b2));
+    a.bc1 = float(1.0 - p1);
+    a.bc2 = float(1.0 - p2);
+    a.lr = lr;
+    a.eps = eps;
+    a.rbc1 = float(1.0 / double(a.bc1));
+    a.rbc2 = float(1.0 / double(a.bc2));
+    a.mhi = a.bc1 * (eps < 0x1p-50f ? eps * 0x1p78f : 0x1p28f);
+    a.vhi = a.bc2 * 0x1p42f;
+    if (a.bc1 >= 0x1p-24f && a.bc2 >= 0x1p-24f)
+        a.newton = (eps <= 0x1p60f ? kNewton : 0) | (eps >= 0x1p-126f && eps <= 0x1p20f ? kNewtonSparse : 0) |
+                   (a.bc1 == 1.f ? kNewtonLowM : 0) | (a.bc2 == 1.f ? kNewtonLowV : 0);
+    return a;
+}
 
 struct SgdmScalars {
     float mu, lr;

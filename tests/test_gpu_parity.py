@@ -201,6 +201,89 @@ def test_adamw_over_the_whole_range_bitexact(n, hp):
         run.close()
 
 
+def _sparse(rng, d, kind):
+    """True where no gradient arrives: scattered elements, or whole rows of 256."""
+    return rng.random(d) < 0.1 if kind == "scattered" else np.repeat(rng.random(-(-d // 256)) < 0.9, 256)[:d]
+
+
+@pytest.mark.parametrize("fused", [False, True], ids=["unfused", "fused"])
+@pytest.mark.parametrize("n", [2, 8])
+@pytest.mark.parametrize("kind", ["scattered", "rows"])
+@pytest.mark.parametrize("start,b2", [(0, 0.95), (400, 0.95), (1200, 0.999)])
+def test_adamw_sparse_moments_bitexact(start, b2, kind, n, fused):
+    """Parameters that get no gradient: moments that are zero, that decay, or that have ended as denormals, before and
+    after the bias corrections have become 1 (round `start`); model elements of 0 and -0 show the quotient's sign."""
+    d, tau = 1 << 14, 2
+    rng = np.random.default_rng(start + n)
+    hp = dataclasses.replace(ADAMW, b2=b2, grad_dtype=W.BF16, flags=W.FLAG_FUSED_ROUND if fused else 0)
+    tensors = (W.Tensor("t", d - 5000, W.KIND_WEIGHT, 1e-3), W.Tensor("u", 5000, W.KIND_WEIGHT, 1e-3, wd=0))
+    x0 = (rng.standard_normal(d) * 0.02).astype(np.float32)
+    x0[rng.random(d) < 0.1] = 0.0
+    x0[rng.random(d) < 0.1] = -0.0
+    run = dsm.DistributedSignMomentum(tensors, n, tau, hp, x0=torch.from_numpy(x0))
+    ora = O.OracleRun(tensors, n, tau, hp, x0=x0)
+    dsm.dsm_set_round(run.h, start)
+    ora.t = start
+    off = _sparse(rng, d, kind)
+    for i in range(n):
+        m = (rng.standard_normal(d) * 1e-3).astype(np.float32)
+        v = (m * m).astype(np.float32)
+        gone = off & (rng.random(d) < 0.5)          # half of them never had a gradient
+        exps = np.repeat(rng.integers(-149, -90, d // 4), 4)
+        m[off], v[off] = (np.float32(2.0) ** exps * rng.uniform(1, 2, d)).astype(np.float32)[off], 0.0
+        if start:
+            some = off & (rng.random(d) < 0.5)
+            v[some] = (np.float32(2.0) ** np.maximum(2 * (exps + 90) - 40, -149)).astype(np.float32)[some]
+        m[gone], v[gone] = 0.0, 0.0
+        m *= rng.choice([-1, 1], d).astype(np.float32)
+        run.write(dsm.BUF_OPT_M, torch.from_numpy(m), worker=i)
+        run.write(dsm.BUF_OPT_V, torch.from_numpy(v), worker=i)
+        ora.opt_m[i][:], ora.opt_v[i][:] = m, v
+    for _ in range(tau):
+        grads = []
+        for i in range(n):
+            g = torch.from_numpy((rng.standard_normal(d) * 1e-3).astype(np.float32) * ~off).bfloat16()
+            run.grad_view(i).copy_(g)
+            grads.append(g.float().numpy())
+        run.local_step()
+        ora.local_step(grads)
+    run.global_step()
+    ora.global_step()
+    compare_state(run, ora, grads=False)
+    run.close()
+
+
+def test_adamw_step_without_gradients_costs_no_more():
+    """A tenth of the elements without a gradient, or nine tenths of the rows: the step reads and writes the same bytes
+    and takes about the time (it took twice as long when a zero moment sent its group to the IEEE divisions)."""
+    d, n = 16_000_000, 2
+    run = dsm.DistributedSignMomentum((W.Tensor("t", d, W.KIND_WEIGHT, 1e-3),), n, 1 << 20,
+                                      dataclasses.replace(ADAMW, grad_dtype=W.BF16))
+    keep = {"dense": torch.ones(d, device="cuda"), "scattered": (torch.rand(d, device="cuda") >= 0.1).float(),
+            "rows": (torch.rand(d // 1000, device="cuda") >= 0.9).repeat_interleave(1000).float()}
+    took = {}
+    for kind in keep:
+        run.write(dsm.BUF_X, torch.zeros(d, device="cuda"))
+        for i in range(n):
+            run.write(dsm.BUF_OPT_M, torch.zeros(d, device="cuda"), worker=i)
+            run.write(dsm.BUF_OPT_V, torch.zeros(d, device="cuda"), worker=i)
+            run.grad_view(i).copy_(torch.randn(d, device="cuda") * 1e-3 * keep[kind])
+        for _ in range(3):
+            run.local_step()
+        best = float("inf")
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                run.local_step()
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        took[kind] = best
+    run.close()
+    assert took["scattered"] < 1.4 * took["dense"] and took["rows"] < 1.4 * took["dense"], took
+
+
 @pytest.mark.parametrize("mode", [W.GLOBAL_SIGN_MOMENTUM, W.GLOBAL_ADAMW], ids=["sign", "gadamw"])
 @pytest.mark.parametrize("n,fused", [(3, False), (4, False), (3, True), (7, True), (8, True), (11, False), (20, False)])
 def test_global_step_over_the_whole_range_bitexact(n, fused, mode):
