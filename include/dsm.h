@@ -306,9 +306,10 @@ int dsm_local_step(dsm_handle* h, dsm_stream_t stream);
  * enqueued on stream before the call; work enqueued on stream after the
  * call follows every copy and every update.  copy_stream may equal stream
  * (no overlap).  Same results, bit for bit, as dsm_load_grads followed by
- * dsm_local_step; where the copies overlap nothing (one chunk, or
- * copy_stream equal to stream) the fused round's last step only enqueues
- * them and leaves the update to dsm_global_step, as dsm_local_step does.
+ * dsm_local_step; where the copies would hide nothing (one chunk, or up to
+ * five for SGD-momentum, or copy_stream equal to stream) the fused round's
+ * last step only enqueues them, up to five chunks in one piece, and leaves
+ * the update to dsm_global_step, as dsm_local_step does.
  * The first call creates the handle's chunk events (cudaEventCreate); the
  * environment variable DSM_HOST_GRAD_CHUNK_BYTES, read then, sets another
  * chunk size.  src must stay unchanged until the copies have completed (until

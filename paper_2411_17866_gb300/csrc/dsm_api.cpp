@@ -626,8 +626,14 @@ int dsm_local_step_host_grads(dsm_handle* h, const void* src, dsm_stream_t strea
     // The fused round's last update would wait for the last copy before it starts; chunk by chunk it runs
     // while the copies do, and only the last chunk's and the global step are left after them (two steps on 16.3 M
     // parameters as above: 1591 -> 1449 us).  A single chunk, or copies without a stream of their own, overlap
-    // nothing, and the update runs inside dsm_global_step as after dsm_local_step.
-    const bool defer = h->fused && h->k + 1 == h->tau && (cs == s || h->ev_copied.size() < 2);
+    // nothing, and the update runs inside dsm_global_step as after dsm_local_step, few chunks copied in one piece.
+    //   SGD-momentum, whose update inside the global step costs little more than the global step alone, needs about
+    // 100 MB of copies to hide the separate one's bytes (rounds of one step, fp32, deferred / chunk by chunk, us: n = 1,
+    // 18 MB 118 / 124, 34 MB 212 / 220, 70 MB 421 / 429, 200 MB 1197 / 1165; n = 4, 34 MB 214 / 227; n = 8, bf16, 18 MB
+    // 126 / 135).
+    constexpr size_t kSgdmChunks = 6;
+    const bool sgdm = h->hp.base == DSM_BASE_SGDM;
+    const bool defer = h->fused && h->k + 1 == h->tau && (cs == s || h->ev_copied.size() < (sgdm ? kSgdmChunks : 2));
     const size_t es = h->al.grad_esize;
     char* grad = static_cast<char*>(h->prob.grad);
     const char* host = static_cast<const char*>(src);
@@ -636,9 +642,10 @@ int dsm_local_step_host_grads(dsm_handle* h, const void* src, dsm_stream_t strea
     cudaError_t err = cudaEventRecord(h->ev_entry, s);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(cs, h->ev_entry, 0);
     if (err != cudaSuccess) return cuda_fail(err, "order the gradient copies after the stream");
-    const uint32_t chunks = static_cast<uint32_t>(h->ev_copied.size());
+    const bool one_piece = defer && h->ev_copied.size() < kSgdmChunks && h->al.d * es < (1ull << 31);
+    const uint32_t chunks = one_piece ? 1 : static_cast<uint32_t>(h->ev_copied.size());
     for (uint32_t c = 0; c < chunks; ++c) {
-        const uint32_t t0 = h->chunk_tile[c], t1 = h->chunk_tile[c + 1];
+        const uint32_t t0 = h->chunk_tile[c], t1 = one_piece ? h->al.num_tiles : h->chunk_tile[c + 1];
         const uint64_t e0 = h->tiles[t0].start + h->tiles[t0].skip(), e1 = h->tiles[t1 - 1].start + h->tiles[t1 - 1].end();
         err = cudaMemcpy2DAsync(grad + e0 * es, h->al.d_stride * es, host + e0 * es, h->al.d * es, (e1 - e0) * es,
                                 h->n, cudaMemcpyHostToDevice, cs);

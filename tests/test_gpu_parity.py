@@ -963,6 +963,28 @@ def test_host_gradient_steps_bitexact(layout_name, name, hp, n, tau, chunk_bytes
     run.close()
 
 
+@pytest.mark.parametrize("chunks", [2, 5, 6])
+def test_host_gradient_steps_sgdm_few_chunks(chunks, monkeypatch):
+    """A fused round of SGD-momentum leaves its last update to the global step up to five chunks, whose gradients it
+    copies in one piece, and updates chunk by chunk from six on."""
+    n, tau = 3, 2
+    d = sum(t.numel for t in RAGGED)
+    monkeypatch.setenv("DSM_HOST_GRAD_CHUNK_BYTES", str(-(-n * d * 4 // chunks)))
+    hp = dataclasses.replace(SGDM, flags=W.FLAG_FUSED_ROUND)
+    run, ora = dsm.DistributedSignMomentum(RAGGED, n, tau, hp), O.OracleRun(RAGGED, n, tau, hp)
+    rng, copy_stream, keep = np.random.default_rng(chunks), torch.cuda.Stream(), []
+    for _ in range(2):
+        for _ in range(tau):
+            g = (rng.standard_normal((n, d)) * 1e-3).astype(np.float32)
+            keep.append(torch.from_numpy(g).pin_memory())
+            run.local_step_host_grads(keep[-1], copy_stream=copy_stream)
+            ora.local_step([g[i] for i in range(n)])
+        run.global_step()
+        ora.global_step()
+        compare_state(run, ora, grads=False)
+    run.close()
+
+
 def test_host_gradient_steps_mix_with_device_fills():
     """Host-gradient steps interleaved with synthetic fills and plain local steps on the same handle."""
     tensors, n, tau = RAGGED, 3, 3
