@@ -34,6 +34,7 @@ int fail(int code, const char* fmt, ...) {
 }
 
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();  // reported here: it must not be found again by a later call's check
     return fail(DSM_ECUDA, "%s: %s (%s)", what, cudaGetErrorString(e), cudaGetErrorName(e));
 }
 
@@ -419,10 +420,7 @@ int dsm_create(const dsm_layout* layout, uint32_t n, uint32_t tau, const dsm_hpa
 
     cudaPointerAttributes attr;
     cudaError_t err = cudaPointerGetAttributes(&attr, dev_arena);
-    if (err != cudaSuccess) {
-        cudaGetLastError();
-        return cuda_fail(err, "cudaPointerGetAttributes(arena)");
-    }
+    if (err != cudaSuccess) return cuda_fail(err, "cudaPointerGetAttributes(arena)");
     if (attr.type != cudaMemoryTypeDevice && attr.type != cudaMemoryTypeManaged)
         return fail(DSM_EALIGN, "arena %p is not device memory", dev_arena);
 

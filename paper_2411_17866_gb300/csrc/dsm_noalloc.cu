@@ -118,6 +118,7 @@ int na_fail(int code, const char* msg) {
 }
 
 int na_cuda(cudaError_t e, const char* what) {
+    cudaGetLastError();  // reported here: it must not be found again by a later call's check
     char buf[512];
     snprintf(buf, sizeof buf, "dsm_global_step_noalloc: %s: %s", what, cudaGetErrorString(e));
     set_last_error_message(buf);
@@ -131,7 +132,6 @@ int check_device_buffer(const void* p, int dev, const char* name) {
     cudaPointerAttributes attr;
     const cudaError_t err = cudaPointerGetAttributes(&attr, p);
     if (err != cudaSuccess) {
-        cudaGetLastError();
         char what[96];
         snprintf(what, sizeof what, "cudaPointerGetAttributes(%s)", name);
         return na_cuda(err, what);

@@ -336,6 +336,29 @@ def test_captured_round_bitexact(n, fused):
     run.close()
 
 
+def test_failed_launch_is_reported_once():
+    """A launch on a stream whose capture has been invalidated (by a wait for it) is refused on the host; the error is
+    that call's alone, and the next one, a new handle here, succeeds."""
+    run = dsm.DistributedSignMomentum(RAGGED, 2, 2, ADAMW)
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        graph.capture_begin(capture_error_mode="thread_local")
+        with pytest.raises(RuntimeError):
+            stream.synchronize()
+        with pytest.raises(dsm.DsmError) as e:
+            run.local_step(stream)
+        assert e.value.code == dsm.DSM_ECUDA
+        with pytest.raises(RuntimeError):
+            graph.capture_end()
+    again, ora = dsm.DistributedSignMomentum(RAGGED, 2, 2, ADAMW), O.OracleRun(RAGGED, 2, 2, ADAMW)
+    ora.run_round()
+    for r in (run, again):      # the refused call left its handle as it was
+        r.synthetic_round()
+        compare_state(r, ora)
+        r.close()
+
+
 @pytest.mark.parametrize("mode", [W.GLOBAL_SIGN_MOMENTUM, W.GLOBAL_ADAMW], ids=["sign", "gadamw"])
 @pytest.mark.parametrize("n", [9, 15, 17, 24, 32, 33, 63, 64])
 def test_many_workers_bitexact(n, mode):
