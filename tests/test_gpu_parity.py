@@ -288,7 +288,8 @@ def test_adamw_step_without_gradients_costs_no_more():
 @pytest.mark.parametrize("n,fused", [(3, False), (4, False), (3, True), (7, True), (8, True), (11, False), (20, False)])
 def test_global_step_over_the_whole_range_bitexact(n, fused, mode):
     """Worker models of every magnitude around x = 0 (the local step leaves them as they are: no gradient, no momentum):
-    the average's and the global AdamW's branch-free divisions inside and outside their ranges."""
+    the average (a product with 1/n where n is a power of two, a division otherwise) and the global step from denormal
+    to overflowing sums."""
     d = 1 << 14
     rng = np.random.default_rng(n)
     hp = dataclasses.replace(SGDM, mu=0.0, sign_mode=W.SIGN, global_mode=mode, flags=W.FLAG_FUSED_ROUND if fused else 0)
@@ -310,6 +311,43 @@ def test_global_step_over_the_whole_range_bitexact(n, fused, mode):
         same_but_for_nan(run.read(which).numpy(), want, what)
     if mode == W.GLOBAL_ADAMW:
         same_but_for_nan(run.read(dsm.BUF_GLOBAL_V).numpy(), ora.gv, "global v")
+    run.close()
+
+
+@pytest.mark.parametrize("n,fused", [(1, False), (3, False), (8, False), (2, True), (8, True), (9, False), (32, False),
+                                     (64, False)])
+def test_statistics_counts_with_nan_and_infinities(n, fused):
+    """The counts for replicas with NaN, both infinities, zeros and sums that vanish: whether the signs agree is taken
+    from the smallest and the largest difference, and fminf and fmaxf pass over NaN."""
+    d = 4096 + 5
+    rng = np.random.default_rng(n)
+    hp = dataclasses.replace(SGDM, mu=0.0, sign_mode=W.SIGN, flags=W.FLAG_FUSED_ROUND if fused else 0)
+    tensors = (W.Tensor("t", 3000, W.KIND_WEIGHT, 1e-3), W.Tensor("u", d - 3000, W.KIND_WEIGHT, 1e-3))
+    x0 = np.zeros(d, np.float32)
+    run = dsm.DistributedSignMomentum(tensors, n, 1, hp, x0=torch.from_numpy(x0))
+    ora = O.OracleRun(tensors, n, 1, hp, x0=x0, with_stats=True)
+    special = np.float32([np.nan, np.inf, -np.inf, 0.0, -0.0, 1e-45, -1e-45, 3e38, -3e38])
+    side = rng.choice([-1.0, 1.0], d)   # every worker on one side, but for
+    kind = rng.integers(0, 4, d)        # 1: one special value, 2: one for each worker, 3: the same for all
+    for i in range(n):
+        v = (side * rng.uniform(1e-3, 1, d)).astype(np.float32)
+        own = special[rng.integers(0, special.size, d)]
+        v = np.where((kind == 2) | ((kind == 1) & (rng.integers(0, n, d) == 0)), own, v)
+        v = np.where(kind == 3, special[np.arange(d) % special.size], v).astype(np.float32)
+        run.write(dsm.BUF_REPLICA, torch.from_numpy(v), worker=i)
+        ora.X[i][:] = v
+    with np.errstate(all="ignore"):
+        run.local_step()
+        ora.local_step([np.zeros(d, np.float32)] * n)
+        stats = run.global_step(with_stats=True)
+        ora.global_step()
+    for T, (got, want) in enumerate(zip(stats, ora.last_stats)):
+        for key in ("zero_sign", "flips", "unanimous", "clamped"):
+            assert got[key] == want[key], (T, key, got[key], want[key])
+        for key in ("delta_sq", "drift"):
+            assert np.isfinite(got[key]) == np.isfinite(want[key]), (T, key, got[key], want[key])
+    same_but_for_nan(run.read(dsm.BUF_X).numpy(), ora.x, "x")
+    same_but_for_nan(run.read(dsm.BUF_M).numpy(), ora.m, "m")
     run.close()
 
 
