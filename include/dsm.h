@@ -455,7 +455,7 @@ const char* dsm_last_error(void);
  * returns. */
 #define DSM_NOALLOC_MAX_TENSORS 4096u
 #define DSM_NOALLOC_MAX_TILES   524288u
-#define DSM_NOALLOC_SCRATCH_BYTES 25657344u
+#define DSM_NOALLOC_SCRATCH_BYTES 25559040u
 int dsm_global_step_noalloc(const dsm_layout* layout, uint32_t n, const dsm_hparams* hp, float gamma,
                             uint64_t round, float* x, float* m, float* replicas, uint64_t replica_stride,
                             dsm_tensor_stats* stats, int stats_is_device, dsm_stream_t stream);

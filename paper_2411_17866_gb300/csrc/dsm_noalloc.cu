@@ -19,9 +19,8 @@ constexpr uint64_t align256(uint64_t v) { return (v + 255) / 256 * 256; }
 
 constexpr uint32_t kNaMaxTensors = DSM_NOALLOC_MAX_TENSORS;
 constexpr uint32_t kNaMaxTiles = DSM_NOALLOC_MAX_TILES;
-// Regions of the scratch array (byte offsets); the first, 24 bytes a tensor, is not used.
-constexpr uint64_t kOffLayout = 0;
-constexpr uint64_t kOffTensors = align256(kOffLayout + sizeof(dsm_tensor) * kNaMaxTensors);
+// Regions of the scratch array (byte offsets).
+constexpr uint64_t kOffTensors = 0;
 constexpr uint64_t kOffTiles = align256(kOffTensors + sizeof(TensorDesc) * kNaMaxTensors);
 constexpr uint64_t kOffPartials = align256(kOffTiles + sizeof(TileDesc) * uint64_t(kNaMaxTiles));
 constexpr uint64_t kOffStats = align256(kOffPartials + sizeof(StatPartial) * uint64_t(kNaMaxTiles));
