@@ -43,7 +43,11 @@ cudaError_t query_fused_shape(const Problem& p, const TensorDesc* tensors, Launc
     // between; n = 4, 1.6 M 49.3 / 46.6, 1.9 M 63.7 / 61.4, 2.2 M 76.0 / 76.0, 3 M 102 / 104; n = 2, 3 M 49.1 / 46.8,
     // 3.7 M 67.7 / 69.0).  Not so n = 1, n >= 5, SGD-momentum and the global AdamW step.
     // Nor where more than a third of the tiles end a CTA's run of one tensor, each with a reduction of its statistics
-    // that the other CTAs of the SM run on through (29.8 M in 174 tensors, n = 4, bf16 gradients: 933 / 915).
+    // that the other CTAs of the SM run on through.  Models of equal tensors, by the share of such tiles, 2 / 3 CTAs:
+    // n = 2, 60 M, bf16 gradients 0.6 1047 / 1005, 0.34 993 / 978, 0.25 978 / 987, 0.15 959 / 987; n = 4, 30 M, bf16
+    // 0.6 889 / 875, 0.34 873 / 877, 0.25 882 / 890; n = 4, 120 M, bf16 0.5 3555 / 3554, 0.34 3518 / 3560; n = 4, 30
+    // M, fp32 1.0 985 / 967, 0.6 927 / 942.
+    // (The line in bytes lies a little above L2, 129 MB, between the sizes above.)
     const uint64_t bytes = p.d_stride * (uint64_t(p.n) * (12 + (p.grad_bf16 ? 2 : 4)) + 8);
     if (p.opt_v && p.n >= 2 && p.n <= 4 && p.global_mode != 4 && bytes > 150000000ull) {
         const uint32_t two = 2 * static_cast<uint32_t>(out->sms);

@@ -65,8 +65,8 @@ __host__ __device__ constexpr size_t fused_smem(bool adamw, bool bf16, int nw, i
 // CTAs per SM that the registers are for: 3; 2 for the global AdamW step, which needs more of them, from n = 7 on.
 // (Rounds of two steps, us.  4 CTAs of 64 registers for n <= 4: GPT-2 S, SGD-momentum, n = 2 1534 against 1477, n = 4
 // 2886 against 2806; in L2, 1 M parameters, AdamW, n = 4 30.6 against 29.2.  Global AdamW, 16.3 M parameters, bf16
-// gradients, n = 8: 3 CTAs 1004, 2 949; left to itself the compiler took 111-212 registers for n > 4.)  See
-// query_fused_shape() for the CTAs that are launched.
+// gradients, n = 8: 3 CTAs 1004, 2 949; left to itself the compiler took 111-212 registers for n > 4.)  At 80 registers
+// AdamW spills 12 to 24 bytes for n = 8 and up to 4 for n = 7.  See query_fused_shape() for the CTAs that are launched.
 __host__ __device__ constexpr int fused_ctas(int nw, int global) { return global == kGlobalAdamW && nw > 6 ? 2 : 3; }
 
 template <bool kAdamW, bool kBf16, int NW, int kGlobal>

@@ -584,9 +584,12 @@ cudaError_t launch_global(const Problem& p, const LaunchShape& ls, const GlobalS
     *grid_used = static_cast<uint32_t>(tiles);
     if (tiles == 0) return cudaSuccess;
     // For a model so small that a round is its launches the last of K4's CTAs sums the statistics, and K5 is not
-    // launched: up to 8 tiles (rounds of one SGD-momentum step, n = 4, without / with K5: 4.5 k parameters in 6 tensors
-    // 6.8 / 7.5 us; 30 tiles 8.1 / 7.6, 244 tiles 14.4 / 10.1).  Not so in the fused round's kernel, which runs 5%
-    // slower on large models for having that code (GPT-2-shaped 184 M, n = 4: 6085 against 5778 us).
+    // launched: up to 8 tiles.  Rounds of one SGD-momentum step, us, without / with K5 (n = 1, 4, 8, 16, 40): 2 tiles
+    // 5.8 / 6.9, 6.4 / 7.0, 7.0 / 7.6, 9.5 / 9.6, 10.5 / 11.4; 8 tiles 5.8 / 7.0, 6.6 / 7.2, 7.2 / 7.7, 9.0 / 9.6,
+    // 11.6 / 11.9; 10 tiles 6.9 / 7.0, 7.5 / 7.4, 8.6 / 7.8, 9.9 / 9.9, 12.3 / 12.1; 24 tiles 7.5 / 7.0, 7.6 / 7.4,
+    // 8.2 / 8.1, 10.2 / 10.0, 13.0 / 13.1; 244 tiles, n = 4, 14.4 / 10.1.  Between, 4 and 6 tiles gain 2 to 8% but
+    // for n = 8 (2% the other way).  Not so in the fused round's kernel, which runs 5% slower on large models for
+    // having that code (GPT-2-shaped 184 M, n = 4: 6085 against 5778 us).
     constexpr uint32_t kSumStatsTiles = 8;
     Problem q = p;
     q.sum_stats = p.num_tiles <= kSumStatsTiles && p.num_tensors <= 4 * kSumStatsTiles;

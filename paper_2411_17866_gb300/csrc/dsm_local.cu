@@ -171,7 +171,9 @@ cudaError_t query_local_shape(const Problem& p, LaunchShape* out) {
     // (GB300, us a step).  From the replicas, fp32 gradients, GPT-2 S with n = 4: 2071 / 2033 / 2056 / 2111 with 2.75 /
     // 3 / 3.25 / 4 CTAs per SM; bf16: 2010 / 1935 / 1907 / 1954 with 2.75 / 3 / 3.5 / 4.  From x (a round of two steps,
     // 184 M parameters, n = 8) fp32: 11279 / 11060 / 11122 with 3 / 3.5 / 4; bf16: 10764 / 10511 / 10294 / 10639 with
-    // 3 / 3.5 / 4 / 4.5.
+    // 3 / 3.5 / 4 / 4.5.  For more workers the bf16 step varies with the distance of their slices, and no number is
+    // best everywhere: 3 / 3.5 / 4, GPT-2 S n = 8 3893 / 3877 / 3969, n = 16 7811 / 8071 / 8122; GPT-2 M n = 8 11275 /
+    // 11001 / 11740; 184 M n = 8 5801 / 5680 / 5914; 52 M at odd offsets n = 16 3436 / 3329 (3 / 3.5).
     const int adamw_ctas = p.grad_bf16 ? 7 * sms / 2 : 3 * sms, adamw_ctas_from_x = p.grad_bf16 ? 4 * sms : 7 * sms / 2;
     out->grid_adamw = std::min(p.grad_bf16 ? grid_for(k_local_adamw<true, false, false>, sms)
                                            : grid_for(k_local_adamw<false, false, false>, sms), adamw_ctas);
